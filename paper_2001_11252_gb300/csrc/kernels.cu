@@ -322,8 +322,8 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
         for (int c = 1; c < kMaxChan; ++c)
             if (c == ch) chnu = L.chan_nu[c];
     }
-    // u0 coefficients of this line for this leaf: computed at the first
-    // scattering in the leaf, then read from shared memory
+    // u0 coefficients of this line for this temperature: computed at the first
+    // scattering in a leaf of it, then read from shared memory
     U0Coef u0c;
     {
         // after the draw rings of Rng
@@ -511,8 +511,11 @@ __device__ __forceinline__ void advance(const Params& P, const Geo& G, Packet<NL
     if (s.enter) {
         load_cell<NL>(P, G, s.w.leaf, s.cc);
         ++tl.leaf_loads;
-        const double k[3] = {s.kd0, s.kd1, s.kd2};
-        double nu_gas = to_gas(s.nu_enter, beta_of(s.cc, k));
+        double nu_gas = s.nu_enter;
+        if (!at_rest(s.cc)) {
+            const double k[3] = {s.kd0, s.kd1, s.kd2};
+            nu_gas = to_gas(s.nu_enter, beta_of(s.cc, k));
+        }
         x_of_nu(P, s.cc, nu_gas, s.xh, s.xl);
         s.budget = 0.0f;
         s.enter = false;
@@ -579,7 +582,8 @@ __device__ __forceinline__ void advance(const Params& P, const Geo& G, Packet<NL
                 } else {
                     ++tl.cross;
                     s.zero_run = tf > 0.0 ? 0 : s.zero_run + 1;
-                    double nu_ext = to_ext(nu_of_x(P, s.cc, s.xh, s.xl), beta_of(s.cc, k));
+                    double nu_ext = nu_of_x(P, s.cc, s.xh, s.xl);
+                    if (!at_rest(s.cc)) nu_ext = to_ext(nu_ext, beta_of(s.cc, k));
                     move_to_face(p, k, axis, tf, s.w);
                     wrap_periodic(G, p, k);
                     s.p0 = p[0]; s.p1 = p[1]; s.p2 = p[2];
@@ -705,6 +709,7 @@ k_propagate(const __grid_constant__ Params P, PacketsIn in, PacketsOut out, Trac
     const unsigned lane = threadIdx.x & 31u;
     bool have = false, drained = false;
     s.mi = 0;
+    s.cc.T = 0.0f;
     uint32_t iters = 0;
     const unsigned long long t0 = P.limits ? global_ns() : 0ull;
     // batch runs: a lane reserves P.refill consecutive packets per queue grab
