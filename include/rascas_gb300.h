@@ -239,8 +239,8 @@ int rascas_set_lines(rascas_ctx *ctx, const rascas_line *lines, int32_t nline, c
 int rascas_set_physics(rascas_ctx *ctx, const rascas_physics *phys);
 /* Bounded device work.  The persistent kernels of rascas_propagate, _trace,
  * _propagate_noalloc and _propagate_batch, and the peeling kernel, give up
- * once a thread has run max_iterations loop iterations (one walk step per
- * iteration; 0 = no limit, at most 2^32 - 1) or a launch has run
+ * once a thread has run max_iterations loop iterations (at most one walk step
+ * per iteration; 0 = no limit, at most 2^32 - 1) or a launch has run
  * time_limit_s seconds of the GPU's global timer (0 = no limit; checked
  * every 256 iterations).  The call then returns RASCAS_E_TIMEOUT; packets in
  * flight are left unfinished (status RASCAS_PK_ACTIVE where statuses are

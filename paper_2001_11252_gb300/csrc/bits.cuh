@@ -96,6 +96,66 @@ RG_HD int64_t order_key(double t) {
 }
 RG_HD double from_key(int64_t k) { return k >= 0 ? bitsd(k) : bitsd((-k) | INT64_MIN); }
 
+RG_HD uint32_t fbits(float x) {
+#if defined(__CUDA_ARCH__)
+    return __float_as_uint(x);
+#else
+    uint32_t b;
+    std::memcpy(&b, &x, 4);
+    return b;
+#endif
+}
+RG_HD float bitsf(uint32_t b) {
+#if defined(__CUDA_ARCH__)
+    return __uint_as_float(b);
+#else
+    float x;
+    std::memcpy(&x, &b, 4);
+    return x;
+#endif
+}
+
+// Conversions between FP32 and FP64 by shifting the bits, equal to the plain
+// casts (which issue on the FP64 pipe: one conversion holds it for as long as
+// a multiply-add, 16 cycles of an SM per warp).  Values outside the normal
+// FP32 range, zeros and NaNs take the cast.
+// (double)f
+RG_HD double widen(float f) {
+    const uint32_t u = fbits(f), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return bitsd((int64_t)((uint64_t)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)) << 32 | (uint64_t)(u << 29)));
+    return (double)f;
+}
+// (float)d, rounded to nearest even
+RG_HD float narrow(double d) {
+    const uint64_t b = (uint64_t)dbits(d);
+    const uint32_t hi = (uint32_t)(b >> 32);
+    if ((hi & 0x7fffffffu) - 0x38100000u < 0x47d00000u - 0x38100000u) {   // 2^-126 <= |d| < 2^126
+        const uint64_t r = (b & 0x7fffffffffffffffull) + 0x0fffffffull + ((b >> 29) & 1ull);
+        return bitsf((hi & 0x80000000u) | ((uint32_t)(r >> 29) - 0xc0000000u));
+    }
+    return (float)d;
+}
+// |d| rounded towards zero to FP32 where it is in the normal range of FP32
+// (2^-126 <= |d| < 2^126), else 0
+RG_HD float narrow_abs_rz(double d) {
+    const uint64_t b = (uint64_t)dbits(d) & 0x7fffffffffffffffull;
+    const bool ok = (uint32_t)(b >> 32) - 0x38100000u < 0x47d00000u - 0x38100000u;
+    return ok ? bitsf((uint32_t)(b >> 29) - 0xc0000000u) : 0.0f;
+}
+
+// d rounded towards minus infinity to FP32, for d >= 2^-126 a truncation
+RG_HD float narrow_down(double d) {
+    const uint64_t b = (uint64_t)dbits(d);
+    if ((uint32_t)(b >> 32) - 0x38100000u < 0x47d00000u - 0x38100000u) return bitsf((uint32_t)(b >> 29) - 0xc0000000u);
+#if defined(__CUDA_ARCH__)
+    return __double2float_rd(d);
+#else
+    const float f = (float)d;
+    return (double)f > d ? std::nextafterf(f, -INFINITY) : f;
+#endif
+}
+
 // ---------------------------------------------------------------------------
 // FP32 pairs: value = h + l with |l| <= ulp(h) / 2 (Dekker 1971; Knuth's
 // two-sum).  About 44 significant bits.

@@ -158,8 +158,8 @@ struct Rng {
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float voigt_h(float a, double x) {
     double x2d = x * x;
-    float x2 = (float)x2d;
-    float lo = (float)(x2d - (double)x2);
+    float x2 = narrow(x2d);
+    float lo = narrow(x2d - widen(x2));
     float e = expf(-x2) * (1.0f - lo);
     float z = __fdividef(x2 - 0.855f, x2 + 3.42f);
     float q = 0.0f;
@@ -214,8 +214,8 @@ __device__ __forceinline__ float voigt_sel(float a, float xh, float xl) {
 }
 __device__ __forceinline__ float voigt_sel(float a, double x) {
     if constexpr (kFaddeeva) {
-        const float xh = (float)x;
-        return faddeeva_h(a, xh, (float)(x - (double)xh));
+        const float xh = narrow(x);
+        return faddeeva_h(a, xh, narrow(x - widen(xh)));
     } else {
         return voigt_h(a, x);
     }
@@ -583,6 +583,54 @@ __device__ __forceinline__ double inner_distance(const double p[3], const Where&
     return from_key(best);
 }
 
+// FP32 screen of an exact step inside a leaf that does not touch the border:
+// 1 = the interaction comes before every face, 2 = the packet leaves through
+// `axis` at distance tf, before the interaction; 0 = too close to tell (within
+// 8e-6, a sign that rounding turned, or a distance too small for FP32), and
+// the plain expressions decide.  kap_box is the opacity times the box size.
+// The distances t = (face - p)/k carry 5e-7 here (truncation to FP32, the
+// quotient, k as sampled), so 8e-6 separates what it claims to; tf is then the
+// plain (face - p) * (1/k) of the one axis that matters.  That leaves three
+// FP64 subtractions instead of the three reciprocals, three products and two
+// products for the optical depth: near leaf corners, where most steps are
+// exact, the FP64 pipe was 80 % busy.  Sphere of tau0 = 1e6, 5e5 packets x 2000
+// scatterings: 154 -> 135 ms together with the conversions by bit shifts.
+__device__ __forceinline__ int screen_step(const double p[3], const double k[3], const float kf[3], const Where& w,
+                                           float kap_box, float tauf, int& axis, double& tf) {
+    const int c[3] = {w.i, w.j, w.k};
+    constexpr float lo = 1.0f - 0x1p-17f, hi = 1.0f + 0x1p-17f;
+    float t0 = __int_as_float(0x7f800000), t1 = t0;
+    double d0 = 0.0, k0 = 0.0;
+    bool tell = true;
+    axis = 0;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        if (is_zero(k[ax])) continue;
+        const double face = dyadic((uint32_t)(is_pos(k[ax]) ? c[ax] + 1 : c[ax]), w.level);
+        const double d = __dsub_rn(face, p[ax]);
+        const float df = narrow_abs_rz(d);
+        tell = tell && df > 0.0f && (dbits(d) ^ dbits(k[ax])) >= 0;
+        const float t = __fdividef(df, fabsf(kf[ax]));
+        if (t < t0) {
+            t1 = t0;
+            t0 = t;
+            axis = ax;
+            d0 = d;
+            k0 = k[ax];
+        } else {
+            t1 = fminf(t1, t);
+        }
+    }
+    const float tc = kap_box * t0;
+    if (!tell) return 0;
+    if (tc > tauf * hi) return 1;
+    if (tc < tauf * lo && t0 < t1 * lo) {
+        tf = __dmul_rn(d0, __drcp_rn(k0));
+        return 2;
+    }
+    return 0;
+}
+
 // move to the exit face along `axis` and snap the crossing coordinate
 __device__ __forceinline__ void move_to_face(double p[3], const double k[3], int axis, double t,
                                              const Where& w) {
@@ -665,37 +713,37 @@ __device__ __forceinline__ void load_cell(const Params& P, const Geo& G, int lea
 // gas-frame frequency from the line-0 Doppler offset x = xh + xl, and back
 template <int NL>
 __device__ __forceinline__ double nu_of_x(const Params& P, const CellCache<NL>& cc, float xh, float xl) {
-    return __fma_rn((double)xh + (double)xl, cc.dnu0, P.line[0].nu0);
+    return __fma_rn(widen(xh) + widen(xl), cc.dnu0, P.line[0].nu0);
 }
 template <int NL>
 __device__ __forceinline__ void x_of_nu(const Params& P, const CellCache<NL>& cc, double nu, float& xh, float& xl) {
     double x = (nu - P.line[0].nu0) * cc.invdnu[0];
-    xh = (float)x;
-    xl = (float)(x - (double)xh);
+    xh = narrow(x);
+    xl = narrow(x - widen(xh));
 }
 
-// total opacity (cm^-1) at the line-0 Doppler offset x = xh + xl; per-line
-// opacities in kl[], each line's own Doppler offset (FP32) in xin[]
+// total opacity (cm^-1) at the line-0 Doppler offset x = xh + xl; cum[i] = the
+// opacity of the dust and of the lines up to i, xin[] = each line's own Doppler
+// offset (FP32).  The multiply-adds are written out: a packet's history depends
+// on their rounding, which must not change with the code around them.
 template <int NL>
 __device__ __forceinline__ float opacity_x(const Params& P, const CellCache<NL>& cc, float xh, float xl,
-                                           float kl[NL], float xin[NL]) {
-    kl[0] = cc.kap0[0] * voigt_sel(cc.a[0], xh, xl);
+                                           float cum[NL], float xin[NL]) {
+    cum[0] = __fmaf_rn(cc.kap0[0], voigt_sel(cc.a[0], xh, xl), cc.kap_d);
     xin[0] = xh;
-    float tot = cc.kap_d + kl[0];
 #pragma unroll
     for (int i = 1; i < NL; ++i) {
-        double x = __fma_rn((double)xh + (double)xl, cc.xb[i], cc.xa[i]);
-        xin[i] = (float)x;
-        kl[i] = cc.kap0[i] * voigt_sel(cc.a[i], x);
-        tot += kl[i];
+        double x = __fma_rn(widen(xh) + widen(xl), cc.xb[i], cc.xa[i]);
+        xin[i] = narrow(x);
+        cum[i] = __fmaf_rn(cc.kap0[i], voigt_sel(cc.a[i], x), cum[i - 1]);
     }
-    return tot;
+    return cum[NL - 1];
 }
 
 // beta = k . v / c in FP64
 template <int NL>
 __device__ __forceinline__ double beta_of(const CellCache<NL>& cc, const double k[3]) {
-    return __fma_rn(k[0], (double)cc.vx, __fma_rn(k[1], (double)cc.vy, k[2] * (double)cc.vz)) * (1.0 / kC);
+    return __fma_rn(k[0], widen(cc.vx), __fma_rn(k[1], widen(cc.vy), k[2] * widen(cc.vz))) * (1.0 / kC);
 }
 
 // gas at rest: beta is 0 and both frame changes are exact identities

@@ -244,9 +244,12 @@ __device__ __forceinline__ bool peel_step(const Params& P, Ray<NL>& r, bool grad
 template <int NL>
 __device__ __forceinline__ void peel_emit(const Params& P, Packet<NL>& s, int d, float wt, double nu_o_gas,
                                           Tallies& tl) {
-    const double b = __fma_rn(P.dirs[d][0], (double)s.cc.vx,
-                              __fma_rn(P.dirs[d][1], (double)s.cc.vy, P.dirs[d][2] * (double)s.cc.vz)) * (1.0 / kC);
-    const double nu_ext = to_ext(nu_o_gas, b);
+    double nu_ext = nu_o_gas;
+    if (!at_rest(s.cc)) {
+        const double b = __fma_rn(P.dirs[d][0], widen(s.cc.vx),
+                                  __fma_rn(P.dirs[d][1], widen(s.cc.vy), P.dirs[d][2] * widen(s.cc.vz))) * (1.0 / kC);
+        nu_ext = to_ext(nu_o_gas, b);
+    }
     const unsigned m = __activemask();
     const int lane = (int)(threadIdx.x & 31u), leader = __ffs(m) - 1;
     unsigned long long base = 0;
@@ -282,7 +285,7 @@ __device__ __forceinline__ void scatter_dust(const Params& P, Packet<NL>& s, Tal
 #pragma unroll
         for (int d = 0; d < kMaxDirs; ++d) {
             if (d < P.ndir) {
-                float muo = s.kx * (float)P.dirs[d][0] + s.ky * (float)P.dirs[d][1] + s.kz * (float)P.dirs[d][2];
+                float muo = s.kx * P.dir_kp[d][0][0] + s.ky * P.dir_kp[d][1][0] + s.kz * P.dir_kp[d][2][0];
                 float wt = phase_p(PH_HG, muo, P.dust_g) * (1.0f / kTwoPiF);
                 peel_emit<NL>(P, s, d, wt, nu_gas, tl);
             }
@@ -290,7 +293,7 @@ __device__ __forceinline__ void scatter_dust(const Params& P, Packet<NL>& s, Tal
     }
     if (!P.keep_dir) {
         dir_from(s.kx, s.ky, s.kz, mu, st, r_phi, s.kx, s.ky, s.kz);
-        s.kd0 = (double)s.kx; s.kd1 = (double)s.ky; s.kd2 = (double)s.kz;
+        s.kd0 = widen(s.kx); s.kd1 = widen(s.ky); s.kd2 = widen(s.kz);
     }
     ++tl.scatt_dust;
 }
@@ -384,16 +387,16 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
 #pragma unroll
         for (int d = 0; d < kMaxDirs; ++d) {
             if (d < P.ndir) {
-                float dx = (float)P.dirs[d][0], dy = (float)P.dirs[d][1], dz = (float)P.dirs[d][2];
+                const float dx = P.dir_kp[d][0][0], dy = P.dir_kp[d][1][0], dz = P.dir_kp[d][2][0];
                 float muo = kx * dx + ky * dy + kz * dz;
                 float uo = dx * vx + dy * vy + dz * vz;
                 double nu_o;
                 if (ch > 0) {
-                    nu_o = __fma_rn(chnu, (double)(uo * vthc), chnu);
+                    nu_o = __fma_rn(chnu, widen(uo * vthc), chnu);
                 } else {
                     float rec = (1.0f - muo) * recp;
                     float f = ((uo - upar) * vthc - rec) / (1.0f + rec);
-                    nu_o = __fma_rn(nu_in, (double)f, nu_in);
+                    nu_o = __fma_rn(nu_in, widen(f), nu_in);
                 }
                 float wt = phase_p(kind, muo, 0.0f) * (1.0f / kTwoPiF);
                 peel_emit<NL>(P, s, d, wt, nu_o, tl);
@@ -402,7 +405,7 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
     }
     float uout = ox * vx + oy * vy + oz * vz;
     if (ch > 0) {
-        double nu = __fma_rn(chnu, (double)(uout * vthc), chnu);
+        double nu = __fma_rn(chnu, widen(uout * vthc), chnu);
         x_of_nu(P, s.cc, nu, s.xh, s.xl);
     } else {
         // nu_out = nu_in (1 + f)  <=>  x_out = x_in + (nu0/Delta nu + x_in) f
@@ -412,7 +415,7 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
     }
     if (!P.keep_dir) {
         s.kx = ox; s.ky = oy; s.kz = oz;
-        s.kd0 = (double)ox; s.kd1 = (double)oy; s.kd2 = (double)oz;
+        s.kd0 = widen(ox); s.kd1 = widen(oy); s.kd2 = widen(oz);
     }
     ++tl.scatt_line;
 }
@@ -499,79 +502,116 @@ __device__ __forceinline__ void finish_packet(const Params& P, const Geo& G, con
     }
 }
 
-// one loop iteration for an active packet: enter a leaf if needed, then one
-// walk step -- an interaction inside the leaf, a face crossing, or the
-// escape through the domain border (Sect. 3, Sect. 4.3).  Each phase appears
-// once, so the loop body stays small for the instruction cache.
+// Whether lanes that wait for a rare, long piece of the loop (an exact step, the
+// next packet) get it now: when they are a quarter of the lanes at work, when
+// nobody else is at work, or when they have waited four iterations.  Issued as
+// soon as one lane asks, a piece that one lane in fifty needs per iteration
+// goes out in every second iteration for one or two lanes.  The wait bounds
+// what a packet with a long history can lose.  Measured with the FP32 screen
+// below, sphere of tau0 = 1e6 (5e5 packets x 2000 scatterings): 126 ms issued
+// at once, 117 at an eighth, 107 at a quarter, 103 at a half or with longer
+// waits, which cost the batch of 200 models 6-20 % and short packets 5 %.
+constexpr int kServeShare = 4;
+constexpr unsigned kServeWait = 4;
+__device__ __forceinline__ bool served(unsigned waiting, unsigned working, unsigned& held) {
+    if (working != 0u && kServeShare * __popc(waiting) < __popc(waiting | working) && ++held < kServeWait) return false;
+    held = 0u;
+    return true;
+}
+
+// one loop iteration of the warp, converged on entry; `active`: this lane has
+// a packet in flight.  Enter a leaf if needed, then at most one walk step --
+// an interaction inside the leaf, a face crossing, or the escape through the
+// domain border (Sect. 3, Sect. 4.3).  Each phase appears once, so the loop
+// body stays small for the instruction cache.
 template <int NL, bool PEEL, bool TRACE>
 __device__ __forceinline__ void advance(const Params& P, const Geo& G, Packet<NL>& s, Tallies& tl,
-                                        const TraceOut& tr) {
-    bool evt = false;
-    s.rng.top_up(P);   // the warp is converged here: draw blocks for all lanes at once
-    if (s.enter) {
-        load_cell<NL>(P, G, s.w.leaf, s.cc);
-        ++tl.leaf_loads;
-        double nu_gas = s.nu_enter;
-        if (!at_rest(s.cc)) {
-            const double k[3] = {s.kd0, s.kd1, s.kd2};
-            nu_gas = to_gas(s.nu_enter, beta_of(s.cc, k));
-        }
-        x_of_nu(P, s.cc, nu_gas, s.xh, s.xl);
-        s.budget = 0.0f;
-        s.enter = false;
-        if (PEEL && s.fresh) {
-            // peeling of the isotropic emission (weight 1/4pi per sr)
+                                        const TraceOut& tr, bool active, unsigned& held) {
+    bool evt = false, inter = false, exact = false, need = false, border_leaf = false;
+    float cum[NL], xin[NL];
+    float kap = 0.0f, li_f = 0.0f;
+    double li_d = 0.0;
+    if (active) {
+        s.rng.top_up(P);   // the warp is converged here: draw blocks for all lanes at once
+        if (s.enter) {
+            load_cell<NL>(P, G, s.w.leaf, s.cc);
+            ++tl.leaf_loads;
+            double nu_gas = s.nu_enter;
+            if (!at_rest(s.cc)) {
+                const double k[3] = {s.kd0, s.kd1, s.kd2};
+                nu_gas = to_gas(s.nu_enter, beta_of(s.cc, k));
+            }
+            x_of_nu(P, s.cc, nu_gas, s.xh, s.xl);
+            s.budget = 0.0f;
+            s.enter = false;
+            if (PEEL && s.fresh) {
+                // peeling of the isotropic emission (weight 1/4pi per sr)
 #pragma unroll
-            for (int d = 0; d < kMaxDirs; ++d)
-                if (d < P.ndir)
-                    peel_emit<NL>(P, s, d, 1.0f / (2.0f * kTwoPiF), nu_gas, tl);
+                for (int d = 0; d < kMaxDirs; ++d)
+                    if (d < P.ndir)
+                        peel_emit<NL>(P, s, d, 1.0f / (2.0f * kTwoPiF), nu_gas, tl);
+            }
+            s.fresh = false;
         }
-        s.fresh = false;
-    }
-    if (P.max_steps > 0 && s.nsteps >= P.max_steps) {
-        s.status = RASCAS_PK_CAPPED_;
-        evt = true;
-    } else {
-        ++s.nsteps;
-        float kl[NL], xin[NL];
-        const float kap = opacity_x<NL>(P, s.cc, s.xh, s.xl, kl, xin);
-        const bool border_leaf = (s.cc.flags & kFlagBorder) != 0;
-        bool inter = false, exact = false;
-        float li_f = 0.0f;
-        double li_d = 0.0;
-        if (!border_leaf) {
-            li_f = __fdividef(s.tauf, kap * G.box_cm_f);
-            float dec = __fmaf_ru(li_f, 1.0f + 0x1p-20f, 4e-16f);
-            if (dec < s.budget) {
-                s.budget = __fsub_rd(s.budget, dec);
-                inter = true;
+        if (P.max_steps > 0 && s.nsteps >= P.max_steps) {
+            s.status = RASCAS_PK_CAPPED_;
+            evt = true;
+        } else {
+            kap = opacity_x<NL>(P, s.cc, s.xh, s.xl, cum, xin);
+            border_leaf = (s.cc.flags & kFlagBorder) != 0;
+            need = true;
+            if (!border_leaf) {
+                li_f = __fdividef(s.tauf, kap * G.box_cm_f);
+                float dec = __fmaf_ru(li_f, 1.0f + 0x1p-20f, 4e-16f);
+                if (dec < s.budget) {
+                    s.budget = __fsub_rd(s.budget, dec);
+                    inter = true;
+                    need = false;
+                }
             }
         }
-        if (!inter) {
+    }
+    const unsigned waiting = __ballot_sync(kFull, need);
+    if (waiting != 0u) {
+        // lanes not served come back with the same step in the next iteration
+        if (!served(waiting, __ballot_sync(kFull, inter), held)) need = false;
+    }
+    if (inter || need) {
+        ++s.nsteps;
+        if (need) {
             // exact FP64 step: distances to the faces and the border
             if (s.tau_fresh) {
-                s.tau = (double)s.tauf;
+                s.tau = widen(s.tauf);
                 s.tau_fresh = false;
             }
             const double k[3] = {s.kd0, s.kd1, s.kd2};
-            // 1/k (the direction changes at almost every scattering, so it
-            // is formed here rather than kept)
-            const double inv[3] = {is_zero(k[0]) ? 0.0 : __drcp_rn(k[0]), is_zero(k[1]) ? 0.0 : __drcp_rn(k[1]),
-                                   is_zero(k[2]) ? 0.0 : __drcp_rn(k[2])};
+            const float kf[3] = {s.kx, s.ky, s.kz};
             double p[3] = {s.p0, s.p1, s.p2};
-            int axis;
-            double tf = face_distance(p, k, inv, s.w, axis);
-            double tb = border_leaf ? border_distance(G, p, k, inv) : kInf;
-            bool border = tb <= tf;
-            double l = border ? tb : tf;
-            double tau_cell = __dmul_rn(__dmul_rn((double)kap, l), G.box_cm);
-            if (tau_cell >= s.tau) {
-                li_d = s.tau / __dmul_rn((double)kap, G.box_cm);
+            int axis = 0, seen = 0;
+            double tf = 0.0, l = 0.0;
+            bool border = false;
+            if (!border_leaf) seen = screen_step(p, k, kf, s.w, kap * G.box_cm_f, s.tauf, axis, tf);
+            if (seen == 0) {
+                // 1/k (the direction changes at almost every scattering, so it
+                // is formed here rather than kept)
+                const double inv[3] = {is_zero(k[0]) ? 0.0 : __drcp_rn(k[0]), is_zero(k[1]) ? 0.0 : __drcp_rn(k[1]),
+                                       is_zero(k[2]) ? 0.0 : __drcp_rn(k[2])};
+                tf = face_distance(p, k, inv, s.w, axis);
+                const double tb = border_leaf ? border_distance(G, p, k, inv) : kInf;
+                border = tb <= tf;
+                l = border ? tb : tf;
+            } else {
+                l = tf;
+            }
+            double tau_cell = 0.0;
+            if (seen != 1) tau_cell = __dmul_rn(__dmul_rn(widen(kap), l), G.box_cm);
+            if (seen == 1 || (seen == 0 && tau_cell >= s.tau)) {
+                li_d = s.tau / __dmul_rn(widen(kap), G.box_cm);
                 inter = true;
                 exact = true;
             } else {
                 s.tau = __dsub_rn(s.tau, tau_cell);
-                s.tauf = (float)s.tau;
+                s.tauf = narrow(s.tau);
                 s.path += l;
                 if (border) {
                     s.p0 = __fma_rn(l, k[0], s.p0);
@@ -581,7 +621,7 @@ __device__ __forceinline__ void advance(const Params& P, const Geo& G, Packet<NL
                     evt = true;
                 } else {
                     ++tl.cross;
-                    s.zero_run = tf > 0.0 ? 0 : s.zero_run + 1;
+                    s.zero_run = order_key(tf) > 0 ? 0 : s.zero_run + 1;
                     double nu_ext = nu_of_x(P, s.cc, s.xh, s.xl);
                     if (!at_rest(s.cc)) nu_ext = to_ext(nu_ext, beta_of(s.cc, k));
                     move_to_face(p, k, axis, tf, s.w);
@@ -610,9 +650,9 @@ __device__ __forceinline__ void advance(const Params& P, const Geo& G, Packet<NL
                 s.path += li_d;
                 const double p[3] = {s.p0, s.p1, s.p2};
                 double D = inner_distance(p, s.w);
-                s.budget = __fsub_rd(__double2float_rd(D * (1.0 - 0x1p-20)), 4e-16f);
+                s.budget = __fsub_rd(narrow_down(D * (1.0 - 0x1p-20)), 4e-16f);
             } else {
-                const double l = (double)li_f;
+                const double l = widen(li_f);
                 s.p0 = __fma_rn(l, s.kd0, s.p0);
                 s.p1 = __fma_rn(l, s.kd1, s.p1);
                 s.p2 = __fma_rn(l, s.kd2, s.p2);
@@ -625,12 +665,8 @@ __device__ __forceinline__ void advance(const Params& P, const Geo& G, Packet<NL
             } else {
                 int il = NL - 1;
 #pragma unroll
-                for (int i = NL - 2; i >= 0; --i) {
-                    float ai = s.cc.kap_d;
-#pragma unroll
-                    for (int j = 0; j <= i; ++j) ai += kl[j];
-                    if (rk < ai) il = i;
-                }
+                for (int i = NL - 2; i >= 0; --i)
+                    if (rk < cum[i]) il = i;
                 if (il == 0) scatter_line<NL, PEEL, 0>(P, G, s, xin[0], tl);
                 if (NL > 1 && il == 1) scatter_line<NL, PEEL, (NL > 1 ? 1 : 0)>(P, G, s, xin[NL > 1 ? 1 : 0], tl);
                 if (NL > 2 && il == 2) scatter_line<NL, PEEL, (NL > 2 ? 2 : 0)>(P, G, s, xin[NL > 2 ? 2 : 0], tl);
@@ -711,6 +747,7 @@ k_propagate(const __grid_constant__ Params P, PacketsIn in, PacketsOut out, Trac
     s.mi = 0;
     s.cc.T = 0.0f;
     uint32_t iters = 0;
+    unsigned held = 0u, idle = 0u;   // iterations that lanes have waited for an exact step, for a packet
     const unsigned long long t0 = P.limits ? global_ns() : 0ull;
     // batch runs: a lane reserves P.refill consecutive packets per queue grab
     long long next = 0, end = 0;
@@ -727,7 +764,10 @@ k_propagate(const __grid_constant__ Params P, PacketsIn in, PacketsOut out, Trac
     for (;;) {
         if (P.limits && out_of_bounds(P, iters, t0)) {
             // a limit was reached: the packet in flight stays unfinished
-            if (have && out.status) out.status[s.idx] = RASCAS_PK_ACTIVE_;
+            if (have && s.status != RASCAS_PK_ACTIVE_)
+                finish_packet<NL>(P, BATCH ? P.models[s.mi] : P.g, s, out, tl);
+            else if (have && out.status)
+                out.status[s.idx] = RASCAS_PK_ACTIVE_;
             break;
         }
         if (PEEL && __any_sync(kFull, have && s.halt)) {
@@ -741,55 +781,59 @@ k_propagate(const __grid_constant__ Params P, PacketsIn in, PacketsOut out, Trac
             if (lane == 0) atomicAdd(P.suspended, 1u);
             break;
         }
-        bool want = !have && !drained;
-        if constexpr (BATCH) {
-            if (want && next < end) {
-                // the next packet of this lane's reservation
-                const long long idx = next++;
-                s.mi = model_of(P, idx);
-                begin_packet<NL, TRACE>(P, P.models[s.mi], in, idx, s, tl, tr);
-                have = true;
-                want = false;
-            }
-        }
-        unsigned m = __ballot_sync(kFull, want);
-        if (m) {
-            int leader = __ffs(m) - 1;
-            const int grab = BATCH ? P.refill : 1;
-            unsigned long long base = 0;
-            if ((int)lane == leader) base = atomicAdd(P.head, (unsigned long long)__popc(m) * grab);
-            base = __shfl_sync(kFull, base, leader);
-            if (want) {
-                long long idx = in.first + (long long)base + (long long)__popc(m & ((1u << lane) - 1u)) * grab;
-                if constexpr (BATCH) {
-                    next = idx + 1;
-                    end = min(idx + grab, in.n);
-                }
-                if (idx < in.n) {
-                    if constexpr (BATCH) {
-                        s.mi = model_of(P, idx);
-                        begin_packet<NL, TRACE>(P, P.models[s.mi], in, idx, s, tl, tr);
-                    } else {
-                        begin_packet<NL, TRACE>(P, P.g, in, idx, s, tl, tr);
-                    }
-                    have = true;
-                } else {
-                    drained = true;
-                }
-            }
-        }
-        if (!__any_sync(kFull, have)) {
-            if (__all_sync(kFull, drained)) break;
-            continue;
-        }
-        if (have) {
-            const Geo& G = BATCH ? P.models[s.mi] : P.g;
-            if (s.status == RASCAS_PK_ACTIVE_) advance<NL, PEEL, TRACE>(P, G, s, tl, tr);
-            if (s.status != RASCAS_PK_ACTIVE_) {
-                finish_packet<NL>(P, G, s, out, tl);
+        // lanes whose packet has ended, or that have none yet, write its
+        // results and take the next one together
+        const bool ended = have && s.status != RASCAS_PK_ACTIVE_;
+        unsigned m = __ballot_sync(kFull, ended || (!have && !drained));
+        if (m && served(m, __ballot_sync(kFull, have && !ended), idle)) {
+            if (ended) {
+                finish_packet<NL>(P, BATCH ? P.models[s.mi] : P.g, s, out, tl);
                 have = false;
             }
+            bool want = !have && !drained;
+            if constexpr (BATCH) {
+                if (want && next < end) {
+                    // the next packet of this lane's reservation
+                    const long long idx = next++;
+                    s.mi = model_of(P, idx);
+                    begin_packet<NL, TRACE>(P, P.models[s.mi], in, idx, s, tl, tr);
+                    have = true;
+                    want = false;
+                }
+            }
+            m = __ballot_sync(kFull, want);
+            if (m) {
+                int leader = __ffs(m) - 1;
+                const int grab = BATCH ? P.refill : 1;
+                unsigned long long base = 0;
+                if ((int)lane == leader) base = atomicAdd(P.head, (unsigned long long)__popc(m) * grab);
+                base = __shfl_sync(kFull, base, leader);
+                if (want) {
+                    long long idx = in.first + (long long)base + (long long)__popc(m & ((1u << lane) - 1u)) * grab;
+                    if constexpr (BATCH) {
+                        next = idx + 1;
+                        end = min(idx + grab, in.n);
+                    }
+                    if (idx < in.n) {
+                        if constexpr (BATCH) {
+                            s.mi = model_of(P, idx);
+                            begin_packet<NL, TRACE>(P, P.models[s.mi], in, idx, s, tl, tr);
+                        } else {
+                            begin_packet<NL, TRACE>(P, P.g, in, idx, s, tl, tr);
+                        }
+                        have = true;
+                    } else {
+                        drained = true;
+                    }
+                }
+            }
+            if (!__any_sync(kFull, have)) {
+                if (__all_sync(kFull, drained)) break;
+                continue;
+            }
         }
+        const Geo& G = BATCH ? P.models[s.mi] : P.g;
+        advance<NL, PEEL, TRACE>(P, G, s, tl, tr, have && s.status == RASCAS_PK_ACTIVE_, held);
     }
     flush(P, tl.pk, CNT_PACKETS);
     flush(P, tl.esc, CNT_ESCAPED);
