@@ -161,10 +161,20 @@ struct Params {
     unsigned int* abort_flag;
     // batch queue: consecutive packets a lane reserves per queue grab
     int refill;
+    // lanes of each warp that take packets (lanes_per_warp)
+    int lanes;
     // run scratch
     unsigned long long* counters;  // [CNT_N]
     unsigned long long* head;      // work-queue head
 };
+
+// Lanes of each warp that work when n items (packets, rays) are shared out over
+// `warps` warps: fewer than 32 where full warps would leave some without any.
+inline int lanes_per_warp(long long n, long long warps) {
+    if (warps < 1) return 32;
+    const long long l = (n + warps - 1) / warps;
+    return l < 1 ? 1 : (l > 32 ? 32 : (int)l);
+}
 
 // words of the counter block: CNT_N counters, the work-queue head, the abort flag
 constexpr int kCounterWords = CNT_N + 2;
