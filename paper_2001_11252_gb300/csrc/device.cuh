@@ -509,6 +509,61 @@ __device__ __forceinline__ bool next_leaf(const Geo& G, const double p[3], const
     return true;
 }
 
+// The same search by the leaf's own links, for the ray walks: the cell across
+// the face comes from one load whose address is known as soon as the leaf is
+// (next_leaf reads the neighbour record, then son, then son again, each after
+// the one before).  The link holds when the target lies in the cell of the
+// leaf's size across the face; a target that rounding has moved past an edge
+// of it, or a link that does not fit, is looked up from the top grid.
+// Against next_leaf: peeling 2^16 packets through the galaxy (2e6 leaves)
+// 55.6 -> 52.4 ms;
+// 2^20 rays no faster, the FP64 pipe bounds them.
+// son_loads and nbor_loads count what next_leaf would have read.
+__device__ __forceinline__ bool linked_leaf(const Geo& G, const double p[3], const double k[3], int axis, Where& w,
+                                            int lk, uint32_t& son_loads, uint32_t& nbor_loads) {
+    const int L = G.max_level, l = w.level, sh = L - l;
+    int t[3];
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) t[ax] = dir_coord(p[ax], k[ax], L);
+    const unsigned n = 1u << L;
+    if ((unsigned)t[0] >= n || (unsigned)t[1] >= n || (unsigned)t[2] >= n) return false;
+    const bool up = is_pos(axis == 0 ? k[0] : (axis == 1 ? k[1] : k[2]));
+    const int step = up ? 1 : -1, wrap = (1 << l) - 1;
+    const int c0 = axis == 0 ? (w.i + step) & wrap : w.i;
+    const int c1 = axis == 1 ? (w.j + step) & wrap : w.j;
+    const int c2 = axis == 2 ? (w.k + step) & wrap : w.k;
+    const int from = axis == 0 ? w.i : (axis == 1 ? w.j : w.k);
+    const bool father = ((from & 1) != 0) != up && l >= 1;   // the cell across the face has the same father
+    const bool holds = (t[0] >> sh) == c0 && (t[1] >> sh) == c1 && (t[2] >> sh) == c2;
+    if (!father && l >= 2) ++nbor_loads;
+    if (!holds || lk == kLinkNone) {
+        uint32_t loads = 0;
+        ++son_loads;
+        return locate(G, t[0], t[1], t[2], w, loads);
+    }
+    if (lk >= 0) {
+        const int coarser = lk & 1;
+        const int s = sh + coarser;
+        son_loads += (father || coarser || l < 2) ? 1u : 2u;
+        w.leaf = lk >> 1;
+        w.level = l - coarser;
+        w.i = t[0] >> s;
+        w.j = t[1] >> s;
+        w.k = t[2] >> s;
+    } else {
+        son_loads += (father || l < 2) ? 1u : 2u;
+        descend(G, -lk, l, 0, t[0], t[1], t[2], w, son_loads);
+    }
+    return true;
+}
+
+// link of leaf w across the exit face of `axis`
+__device__ __forceinline__ int face_link(const Geo& G, const Where& w, const double k[3], int axis) {
+    const bool up = is_pos(axis == 0 ? k[0] : (axis == 1 ? k[1] : k[2]));
+    const int face = 2 * max(axis, 0) + (up ? 1 : 0);   // axis -1: a zero direction, which leaves the box next
+    return __ldg(G.link + 8ll * w.leaf + face);
+}
+
 // distance along k from p to the exit face of leaf w (FP64, exactly the
 // oracle's (face - p) * (1/k)); axis = crossed axis, ties to the lowest axis.
 // Face coordinates, the choice of the minimum and the clamp at zero run on

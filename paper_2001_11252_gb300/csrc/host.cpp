@@ -65,7 +65,7 @@ struct rascas_ctx {
     // mesh
     bool has_mesh = false;
     HostMesh mesh;
-    DevBuf d_rec, d_son, d_nbr, d_top;
+    DevBuf d_rec, d_son, d_nbr, d_top, d_link;
     // problem
     bool has_domain = false, has_lines = false, has_phys = false, has_det = false;
     rascas_domain dom{};
@@ -335,7 +335,7 @@ int rascas_create(rascas_ctx** out, int device) {
 int rascas_destroy(rascas_ctx* ctx) {
     if (!ctx) return RASCAS_E_ARG;
     cudaSetDevice(ctx->device);
-    for (DevBuf* b : {&ctx->d_rec, &ctx->d_son, &ctx->d_nbr, &ctx->d_top, &ctx->d_spec, &ctx->d_pspec,
+    for (DevBuf* b : {&ctx->d_rec, &ctx->d_son, &ctx->d_nbr, &ctx->d_top, &ctx->d_link, &ctx->d_spec, &ctx->d_pspec,
                       &ctx->d_pimg, &ctx->d_pcube, &ctx->d_counters, &ctx->d_params, &ctx->stage_in,
                       &ctx->stage_out, &ctx->stage_aux, &ctx->stage_adj, &ctx->ray_init, &ctx->peel_rec,
                       &ctx->peel_prep, &ctx->peel_live, &ctx->peel_save, &ctx->peel_flag, &ctx->peel_ctl,
@@ -372,6 +372,7 @@ int rascas_load_octree(rascas_ctx* ctx, const rascas_octree* t, int mem) {
     CK(ctx->d_son.ensure(M.son.size() * 4));
     CK(ctx->d_nbr.ensure(M.nbr.size() * 4));
     CK(ctx->d_top.ensure(M.top.size() * 4));
+    CK(ctx->d_link.ensure(M.rec.size() * 4));
     CK(cudaMemcpy(ctx->d_rec.p, M.rec.data(), M.rec.size() * 4, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(ctx->d_son.p, M.son.data(), M.son.size() * 4, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(ctx->d_nbr.p, M.nbr.data(), M.nbr.size() * 4, cudaMemcpyHostToDevice));
@@ -387,6 +388,10 @@ int rascas_load_octree(rascas_ctx* ctx, const rascas_octree* t, int mem) {
     P.g.noct = M.noct;
     P.g.box_cm = M.box_cm;
     P.g.box_cm_f = (float)M.box_cm;
+    // the walk's face links, formed on the device from the records above
+    CK(rg::launch_leaf_links(P.g, (int*)ctx->d_link.p, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    P.g.link = (const int*)ctx->d_link.p;
     ctx->mesh = std::move(M);
     ctx->has_mesh = true;
     return RASCAS_OK;
@@ -1135,6 +1140,7 @@ int rascas_load_batch(rascas_ctx* ctx, const rascas_model* models, int32_t nmode
         CK(cudaMemcpy(dtop, M.top.data(), M.top.size() * 4, cudaMemcpyHostToDevice));
         rg::Geo& G = geo[k];
         G.rec = (const float4*)drec; G.son = (const int*)dson; G.nbr = (const int4*)dnbr; G.top = (const int4*)dtop;
+        G.link = nullptr;
         G.top_level = M.top_level; G.max_level = M.max_level; G.nleaf = M.nleaf; G.noct = M.noct;
         G.box_cm = M.box_cm; G.box_cm_f = (float)M.box_cm;
         G.dom_kind = md.domain.kind;

@@ -10,6 +10,12 @@ constexpr int kMaxLines = 4;
 constexpr int kMaxChan = 4;
 constexpr int kMaxDirs = 8;
 
+// Face links of a leaf, in the order -x, +x, -y, +y, -z, +z (two words pad the
+// record to one 32-byte sector): leaf << 1 | (1 if that leaf is one level
+// coarser), or -oct when the cell across the face is refined, or kLinkNone
+// (more than one level coarser, or a leaf index that does not fit)
+constexpr int kLinkNone = (int)0x80000000;
+
 // per-packet status values (same numbers as RASCAS_PK_* of the C ABI)
 constexpr int RASCAS_PK_ACTIVE_ = 0;
 constexpr int RASCAS_PK_ESCAPED_ = 1;
@@ -57,6 +63,7 @@ struct Geo {
     const int* son;        // [8*noct]
     const int4* nbr;       // [2*noct]: {nb0, nb1, nb2, nb3}, {nb4, nb5, father, packed levels}
     const int4* top;       // [(2^S)^3]: {code, level, oct, 0}
+    const int* link;       // [8*nleaf]: per leaf the cell across each face (kLink...); single-model runs
     int top_level, max_level, nleaf, noct;
     double box_cm;
     float box_cm_f;
@@ -249,6 +256,8 @@ cudaError_t launch_ray_columns(const Params& P, long long n, const double* pos, 
 cudaError_t launch_grad_unpack(long long nleaf, const float4* src, float* dst, cudaStream_t st);
 cudaError_t launch_pack_fields(long long n, const float* nh, const float* vx, const float* vy, const float* vz,
                                const float* T, const float* nd, const float* nm, float4* rec, cudaStream_t st);
+// the face links of every leaf, from the octs' son and neighbour records
+cudaError_t launch_leaf_links(const Geo& g, int* link, cudaStream_t st);
 cudaError_t launch_eval_voigt(long long n, const float* a, const double* x, float* H, int method, cudaStream_t st);
 cudaError_t launch_sample_upar(const Params& P, long long n, const double* x, const float* a,
                                const uint64_t* id, float* u, int32_t* ndraw, cudaStream_t st);

@@ -140,7 +140,7 @@ __device__ __forceinline__ bool ray_step(const Params& P, Ray<NL>& r, float tsto
         border = order_key(tb) <= order_key(tf);
         if (border) l = tb;
     }
-    r.tau = f2_add_f(r.tau, kap * (float)l * P.g.box_cm_f);
+    r.tau = f2_add_f(r.tau, kap * narrow(l) * P.g.box_cm_f);
     if (cells != nullptr && r.n < cap) {
         cells[r.n] = r.w.leaf;
         lens[r.n] = l;
@@ -149,9 +149,10 @@ __device__ __forceinline__ bool ray_step(const Params& P, Ray<NL>& r, float tsto
     if (border || r.tau.h > tstop) return true;
     r.zero_run = order_key(tf) > 0 ? 0 : r.zero_run + 1;
     if (r.zero_run > 64) return true;
+    const int lk = face_link(P.g, r.w, r.k, axis);
     move_to_face(r.p, r.k, axis, tf, r.w);
     wrap_periodic(P.g, r.p, r.k);
-    return !next_leaf(P.g, r.p, r.k, axis, r.w, sl, nl);
+    return !linked_leaf(P.g, r.p, r.k, axis, r.w, lk, sl, nl);
 }
 
 __device__ __forceinline__ float tau_stop_f(double tau_stop) {
@@ -191,7 +192,7 @@ __device__ __forceinline__ void grad_add(const Params& P, const Ray<NL>& r, cons
         // sigma0, a and x all scale as T^(-1/2)
         dk[4] += nX * s0 * (-0.5f / Tm) * (H + a * Ha + x * Hx);
     }
-    const float f = scale * P.g.box_cm_f * (float)l;
+    const float f = scale * P.g.box_cm_f * narrow(l);
     if (f != 0.0f) {
         // the leaf's six derivatives sit in one 32-byte sector: two vector atomics
         float4* g = reinterpret_cast<float4*>(P.adj_grad) + 2 * (long long)r.w.leaf;
@@ -226,15 +227,16 @@ __device__ __forceinline__ bool peel_step(const Params& P, Ray<NL>& r, bool grad
         grad_add<NL>(P, r, r0, r1, xh, beta, l, scale);
         if (border) return true;
     } else {
-        r.tau = f2_add_f(r.tau, kap * (float)l * P.g.box_cm_f);
+        r.tau = f2_add_f(r.tau, kap * narrow(l) * P.g.box_cm_f);
         ++r.n;
         if (border || r.tau.h > tstop) return true;
     }
     r.zero_run = order_key(tf) > 0 ? 0 : r.zero_run + 1;
     if (r.zero_run > 64) return true;
+    const int lk = face_link(P.g, r.w, r.k, axis);
     move_to_face(r.p, r.k, axis, tf, r.w);
     wrap_periodic(P.g, r.p, r.k);
-    return !next_leaf(P.g, r.p, r.k, axis, r.w, sl, nl);
+    return !linked_leaf(P.g, r.p, r.k, axis, r.w, lk, sl, nl);
 }
 
 // one peeling ray towards direction d (weight wt per sr, gas-frame frequency
@@ -918,12 +920,12 @@ __device__ __forceinline__ void ray_load(const RayInit* __restrict__ in, long lo
 template <int NL>
 __global__ void __launch_bounds__(128, 8) k_ray_tau(const Params* __restrict__ G, long long n,
                                                  const RayInit* __restrict__ init, double* tau, int32_t* cells,
-                                                 double* lens, int cap, int32_t* ncell) {
+                                                 double* lens, int cap, int32_t* ncell, int lanes) {
     const Params& P = *G;
     const unsigned lane = threadIdx.x & 31u;
     Ray<NL> r;
     long long i = -1;
-    bool active = false, drained = false;
+    bool active = false, drained = (int)lane >= lanes;
     uint32_t sl = 0, nl = 0, steps = 0;
     const float tstop = __int_as_float(0x7f800000);
     for (;;) {
@@ -1039,7 +1041,7 @@ __device__ __forceinline__ bool first_leaf_dark(const Params& P, const Ray<NL>& 
         border = order_key(tb) <= order_key(tf);
         if (border) l = tb;
     }
-    const f2 tau = f2_add_f(r.tau, kap * (float)l * P.g.box_cm_f);
+    const f2 tau = f2_add_f(r.tau, kap * narrow(l) * P.g.box_cm_f);
     return (border || tau.h > tstop) && !(f2_val(tau) <= P.tau_stop);
 }
 
@@ -1228,7 +1230,7 @@ __device__ __forceinline__ bool col_step(const Params& P, ColRay& r, uint32_t& s
         border = order_key(tb) <= order_key(tf);
         if (border) l = tb;
     }
-    const float lc = (float)l * P.g.box_cm_f;
+    const float lc = narrow(l) * P.g.box_cm_f;
     r.nh = f2_add_f(r.nh, r0.x * lc);
     r.nd = f2_add_f(r.nd, r1.y * lc);
     r.nm = f2_add_f(r.nm, r1.z * lc);
@@ -1236,21 +1238,22 @@ __device__ __forceinline__ bool col_step(const Params& P, ColRay& r, uint32_t& s
     if (border) return true;
     r.zero_run = order_key(tf) > 0 ? 0 : r.zero_run + 1;
     if (r.zero_run > 64) return true;
+    const int lk = face_link(P.g, r.w, r.k, axis);
     move_to_face(r.p, r.k, axis, tf, r.w);
     wrap_periodic(P.g, r.p, r.k);
-    return !next_leaf(P.g, r.p, r.k, axis, r.w, sl, nl);
+    return !linked_leaf(P.g, r.p, r.k, axis, r.w, lk, sl, nl);
 }
 
 // persistent walk over the rays set up by k_ray_prep; the queue head P.head
 // must be zero on entry
 __global__ void __launch_bounds__(128, 8) k_ray_columns(const Params* __restrict__ G, long long n,
                                                      const RayInit* __restrict__ init, double* cols, double* tau,
-                                                     double sig_hi, double sig_d, int32_t* ncell) {
+                                                     double sig_hi, double sig_d, int32_t* ncell, int lanes) {
     const Params& P = *G;
     const unsigned lane = threadIdx.x & 31u;
     ColRay r;
     long long i = -1;
-    bool active = false, drained = false;
+    bool active = false, drained = (int)lane >= lanes;
     uint32_t sl = 0, nl = 0, steps = 0;
     for (;;) {
         const bool want = !active && !drained;
@@ -1305,6 +1308,49 @@ __global__ void __launch_bounds__(128, 8) k_ray_columns(const Params* __restrict
                 active = false;
             }
         }
+    }
+}
+
+// One thread per oct: the face links of its leaves.  Within the oct the cell
+// across a face is a sibling; across the oct's own faces it lies in the
+// father's neighbour cell, which is a leaf one level coarser, the oct of the
+// siblings' level, or (in a tree that is not graded) a coarser leaf still.
+// The root oct's neighbours are its own cells, the box being periodic here
+// (the walk tests the box edge on the coordinates).
+__global__ void k_leaf_links(Geo g, int* __restrict__ link) {
+    const long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (o >= g.noct) return;
+    const int4 a = __ldg(g.nbr + 2 * o), b = __ldg(g.nbr + 2 * o + 1);
+    const int nb[6] = {a.x, a.y, a.z, a.w, b.x, b.y};
+    int level = 1;
+    for (int f = b.z; f >= 0 && level < 32; f = __ldg(g.nbr + 2 * (long long)(f >> 3) + 1).z) ++level;
+    auto code_of = [](int v, int coarser) {   // son value v of the cell across the face
+        if (v > 0) return -v;
+        const int leaf = -v - 1;
+        return leaf < (1 << 30) ? (leaf << 1 | coarser) : kLinkNone;
+    };
+    for (int c = 0; c < 8; ++c) {
+        const int v = __ldg(g.son + 8 * o + c);
+        if (v > 0) continue;
+        int* out = link + 8ll * (-v - 1);
+#pragma unroll
+        for (int face = 0; face < 6; ++face) {
+            const int bit = 1 << (face >> 1);
+            const bool inside = ((c & bit) != 0) != ((face & 1) != 0);
+            int lk;
+            if (inside || level == 1) {
+                lk = code_of(__ldg(g.son + 8 * o + (c ^ bit)), 0);
+            } else {
+                const int nl = (b.w >> (5 * face)) & 31;
+                const int s = nb[face] >= 0 ? __ldg(g.son + (long long)nb[face]) : 0;
+                if (s == 0) lk = kLinkNone;
+                else if (s < 0) lk = nl == level - 1 ? code_of(s, 1) : kLinkNone;
+                else lk = code_of(__ldg(g.son + 8ll * s + (c ^ bit)), 0);
+            }
+            out[face] = lk;
+        }
+        out[6] = level;
+        out[7] = 0;
     }
 }
 
@@ -1437,6 +1483,14 @@ cudaError_t RG_SFX(launch_peel)(const Params& P, int sms, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// n rays go to eight warps per SM first, one lane each, then two lanes each and
+// so on; only from 32 on does the number of warps grow
+static int ray_lanes(long long n, int sms) { return lanes_per_warp(n, (long long)sms * 8); }
+static unsigned ray_grid(long long n, int lanes, int resident, int block) {
+    const long long per_block = (long long)lanes * (block / 32);
+    return (unsigned)std::min<long long>((n + per_block - 1) / per_block, resident);
+}
+
 // the queue head P.head must be zero on entry
 cudaError_t RG_SFX(launch_ray_tau)(const Params& P, long long n, const double* pos, const double* dir, const double* nu,
                            double* tau, int32_t* cells, double* lens, int cap, int32_t* ncell, RayInit* init,
@@ -1446,14 +1500,15 @@ cudaError_t RG_SFX(launch_ray_tau)(const Params& P, long long n, const double* p
     const int per_sm = P.nline == 1 ? ray_occ<1>() : P.nline == 2 ? ray_occ<2>() : P.nline == 3 ? ray_occ<3>()
                                                                                                : ray_occ<4>();
     const long long need = (n + block - 1) / block;
-    const unsigned grid = (unsigned)std::min<long long>(need, (long long)sms * per_sm);
+    const int lanes = ray_lanes(n, sms);
+    const unsigned grid = ray_grid(n, lanes, sms * per_sm, block);
     const unsigned gp = (unsigned)need;
     const Params* G = P.self;
     switch (P.nline) {
 #define RG_RAY(NLV)                                                                          \
     case NLV:                                                                                \
         k_ray_prep<NLV><<<gp, block, 0, st>>>(G, n, pos, dir, nu, init);                     \
-        k_ray_tau<NLV><<<grid, block, 0, st>>>(G, n, init, tau, cells, lens, cap, ncell);    \
+        k_ray_tau<NLV><<<grid, block, 0, st>>>(G, n, init, tau, cells, lens, cap, ncell, lanes); \
         break;
         RG_RAY(1)
         RG_RAY(2)
@@ -1509,9 +1564,15 @@ cudaError_t launch_ray_columns(const Params& P, long long n, const double* pos, 
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ray_columns, block, 0);
     if (per_sm < 1) per_sm = 1;
     const long long need = (n + block - 1) / block;
-    const unsigned grid = (unsigned)std::min<long long>(need, (long long)sms * per_sm);
+    const int lanes = ray_lanes(n, sms);
+    const unsigned grid = ray_grid(n, lanes, sms * per_sm, block);
     k_ray_prep<1><<<(unsigned)need, block, 0, st>>>(P.self, n, pos, dir, nullptr, init);
-    k_ray_columns<<<grid, block, 0, st>>>(P.self, n, init, cols, tau, sig_hi, sig_d, ncell);
+    k_ray_columns<<<grid, block, 0, st>>>(P.self, n, init, cols, tau, sig_hi, sig_d, ncell, lanes);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_leaf_links(const Geo& g, int* link, cudaStream_t st) {
+    k_leaf_links<<<(unsigned)((g.noct + 127) / 128), 128, 0, st>>>(g, link);
     return cudaGetLastError();
 }
 
