@@ -132,7 +132,7 @@ __device__ __forceinline__ bool ray_step(const Params& P, Ray<NL>& r, float tsto
     f2 beta;
     const float kap = ray_opacity<NL>(P, r.R, r0, r1, kl, xh, xl, beta);
     int axis;
-    const double tf = face_distance(r.p, r.k, r.inv, r.w, axis);
+    const double tf = exit_distance(r.p, r.k, r.inv, r.w, axis);
     bool border = false;
     double l = tf;
     if (__float_as_int(r1.w) & kFlagBorder) {
@@ -150,7 +150,7 @@ __device__ __forceinline__ bool ray_step(const Params& P, Ray<NL>& r, float tsto
     r.zero_run = order_key(tf) > 0 ? 0 : r.zero_run + 1;
     if (r.zero_run > 64) return true;
     const int lk = face_link(P.g, r.w, r.k, axis);
-    move_to_face(r.p, r.k, axis, tf, r.w);
+    move_through_face(r.p, r.k, axis, tf, r.w);
     wrap_periodic(P.g, r.p, r.k);
     return !linked_leaf(P.g, r.p, r.k, axis, r.w, lk, sl, nl);
 }
@@ -215,7 +215,7 @@ __device__ __forceinline__ bool peel_step(const Params& P, Ray<NL>& r, bool grad
     f2 beta;
     const float kap = ray_opacity<NL>(P, r.R, r0, r1, kl, xh, xl, beta);
     int axis;
-    const double tf = face_distance(r.p, r.k, r.inv, r.w, axis);
+    const double tf = exit_distance(r.p, r.k, r.inv, r.w, axis);
     bool border = false;
     double l = tf;
     if (__float_as_int(r1.w) & kFlagBorder) {
@@ -234,7 +234,7 @@ __device__ __forceinline__ bool peel_step(const Params& P, Ray<NL>& r, bool grad
     r.zero_run = order_key(tf) > 0 ? 0 : r.zero_run + 1;
     if (r.zero_run > 64) return true;
     const int lk = face_link(P.g, r.w, r.k, axis);
-    move_to_face(r.p, r.k, axis, tf, r.w);
+    move_through_face(r.p, r.k, axis, tf, r.w);
     wrap_periodic(P.g, r.p, r.k);
     return !linked_leaf(P.g, r.p, r.k, axis, r.w, lk, sl, nl);
 }
@@ -914,11 +914,12 @@ __device__ __forceinline__ void ray_load(const RayInit* __restrict__ in, long lo
 
 // Persistent walk: each lane walks one ray leaf by leaf and takes the next ray
 // from the queue head as soon as its ray is done, so the lanes of a warp stay
-// busy whatever the spread of ray lengths. Eight blocks per SM (64 registers,
-// a few spilled values) hide more of the dependent leaf-record loads than the
-// five that the unconstrained register count allows.
+// busy whatever the spread of ray lengths.  Six blocks per SM (80 registers, no
+// spills): 2^20 rays of 153 leaves through the galaxy in 7.6 ms, 7.8 with eight
+// blocks (64 registers); 9.5 ms with next_leaf and face_distance (the walk of
+// the scattering kernel), eight blocks.
 template <int NL>
-__global__ void __launch_bounds__(128, 8) k_ray_tau(const Params* __restrict__ G, long long n,
+__global__ void __launch_bounds__(128, 6) k_ray_tau(const Params* __restrict__ G, long long n,
                                                  const RayInit* __restrict__ init, double* tau, int32_t* cells,
                                                  double* lens, int cap, int32_t* ncell, int lanes) {
     const Params& P = *G;
@@ -1222,7 +1223,7 @@ __device__ __forceinline__ bool col_step(const Params& P, ColRay& r, uint32_t& s
     const float4 r0 = __ldg(P.g.rec + 2 * r.w.leaf);
     const float4 r1 = __ldg(P.g.rec + 2 * r.w.leaf + 1);
     int axis;
-    const double tf = face_distance(r.p, r.k, r.inv, r.w, axis);
+    const double tf = exit_distance(r.p, r.k, r.inv, r.w, axis);
     bool border = false;
     double l = tf;
     if (__float_as_int(r1.w) & kFlagBorder) {
@@ -1239,14 +1240,14 @@ __device__ __forceinline__ bool col_step(const Params& P, ColRay& r, uint32_t& s
     r.zero_run = order_key(tf) > 0 ? 0 : r.zero_run + 1;
     if (r.zero_run > 64) return true;
     const int lk = face_link(P.g, r.w, r.k, axis);
-    move_to_face(r.p, r.k, axis, tf, r.w);
+    move_through_face(r.p, r.k, axis, tf, r.w);
     wrap_periodic(P.g, r.p, r.k);
     return !linked_leaf(P.g, r.p, r.k, axis, r.w, lk, sl, nl);
 }
 
 // persistent walk over the rays set up by k_ray_prep; the queue head P.head
 // must be zero on entry
-__global__ void __launch_bounds__(128, 8) k_ray_columns(const Params* __restrict__ G, long long n,
+__global__ void __launch_bounds__(128, 6) k_ray_columns(const Params* __restrict__ G, long long n,
                                                      const RayInit* __restrict__ init, double* cols, double* tau,
                                                      double sig_hi, double sig_d, int32_t* ncell, int lanes) {
     const Params& P = *G;

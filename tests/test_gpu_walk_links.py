@@ -1,7 +1,7 @@
-"""The ray walks by face links: the leaves
+"""The ray walks by face links with the exit face chosen in FP32: the leaves
 and FP64 path lengths must be the oracle's, bit for bit, on trees where the
 general search is needed (levels that jump by more than one, a one-level
-tree, a periodic slab) and on rays where the choice of the exit face is close (ties
+tree, a periodic slab) and on rays where the FP32 choice cannot tell (ties
 between axes, directions along axes and with components next to zero, starts
 on faces, edges and corners); and a ray's result must not depend on how many
 rays share the launch."""
