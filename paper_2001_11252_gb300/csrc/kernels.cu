@@ -75,20 +75,34 @@ __device__ __forceinline__ void dir_from_basis(float kx, float ky, float kz, con
                                                float mu, float st, float r_phi, float& ox, float& oy, float& oz) {
     float sn, cs;
     sincospif(2.0f * r_phi, &sn, &cs);
-    float x = mu * kx + st * (cs * e1.x + sn * e2.x);
-    float y = mu * ky + st * (cs * e1.y + sn * e2.y);
-    float z = mu * kz + st * (cs * e1.z + sn * e2.z);
-    float nn = rsqrtf(x * x + y * y + z * z);
+    // multiply-adds written out: a history depends on their rounding, which must
+    // not change with the code around them
+    float x = __fmaf_rn(st, __fmaf_rn(sn, e2.x, cs * e1.x), mu * kx);
+    float y = __fmaf_rn(st, __fmaf_rn(sn, e2.y, cs * e1.y), mu * ky);
+    float z = __fmaf_rn(st, __fmaf_rn(cs, e1.z, sn * e2.z), mu * kz);
+    float nn = rsqrtf(__fmaf_rn(z, z, __fmaf_rn(x, x, y * y)));
     ox = x * nn;
     oy = y * nn;
     oz = z * nn;
 }
 
+// the same for dust, with the roundings it has had (other ones with one line
+// than with several)
+template <int NL>
 __device__ __forceinline__ void dir_from(float kx, float ky, float kz, float mu, float st, float r_phi,
                                          float& ox, float& oy, float& oz) {
     float3 e1, e2;
     onb(kx, ky, kz, e1, e2);
-    dir_from_basis(kx, ky, kz, e1, e2, mu, st, r_phi, ox, oy, oz);
+    float sn, cs;
+    sincospif(2.0f * r_phi, &sn, &cs);
+    float x = __fmaf_rn(mu, kx, st * __fmaf_rn(sn, e2.x, cs * e1.x));
+    float y = __fmaf_rn(mu, ky, st * __fmaf_rn(cs, e1.y, sn * e2.y));
+    const float zi = __fmaf_rn(cs, e1.z, sn * e2.z);
+    float z = NL == 1 ? __fmaf_rn(st, zi, mu * kz) : __fmaf_rn(mu, kz, st * zi);
+    float nn = rsqrtf(__fmaf_rn(z, z, NL == 1 ? __fmaf_rn(x, x, y * y) : __fmaf_rn(y, y, x * x)));
+    ox = x * nn;
+    oy = y * nn;
+    oz = z * nn;
 }
 
 // ---------------------------------------------------------------------------
@@ -294,17 +308,18 @@ __device__ __forceinline__ void scatter_dust(const Params& P, Packet<NL>& s, Tal
         }
     }
     if (!P.keep_dir) {
-        dir_from(s.kx, s.ky, s.kz, mu, st, r_phi, s.kx, s.ky, s.kz);
+        dir_from<NL>(s.kx, s.ky, s.kz, mu, st, r_phi, s.kx, s.ky, s.kz);
         s.kd0 = widen(s.kx); s.kd1 = widen(s.ky); s.kd2 = widen(s.kz);
     }
     ++tl.scatt_dust;
 }
 
-// x = xh + xl advanced by d, kept as a normalised FP32 pair (two-sum)
-__device__ __forceinline__ void pair_add(float& xh, float& xl, float d) {
-    float sum = xh + d;
+// x = xh + xl advanced by a f, kept as a normalised FP32 pair (two-sum; the
+// product is not rounded by itself)
+__device__ __forceinline__ void pair_add(float& xh, float& xl, float a, float f) {
+    float sum = __fmaf_rn(a, f, xh);
     float bb = sum - xh;
-    float err = (xh - (sum - bb)) + (d - bb);
+    float err = (xh - (sum - bb)) + __fmaf_rn(a, f, -bb);
     float lo = xl + err;
     float hi = sum + lo;
     xl = lo - (hi - sum);
@@ -333,15 +348,15 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
     {
         // after the draw rings of Rng
         extern __shared__ float s_u0[];
-        float* col = s_u0 + (size_t)(kRing + IL * 6) * blockDim.x + threadIdx.x;
+        float* col = s_u0 + (kRing + IL * 6) * kCols + threadIdx.x;
         if (!(s.cc.u0mask & (1u << IL))) {
             u0_coeffs(L.a_over_invdnu * s.cc.invdnu[IL], u0c);
 #pragma unroll
-            for (int c = 0; c < 6; ++c) col[c * blockDim.x] = u0c.b[c];
+            for (int c = 0; c < 6; ++c) col[c * kCols] = u0c.b[c];
             s.cc.u0mask |= 1u << IL;
         } else {
 #pragma unroll
-            for (int c = 0; c < 6; ++c) u0c.b[c] = col[c * blockDim.x];
+            for (int c = 0; c < 6; ++c) u0c.b[c] = col[c * kCols];
         }
     }
     bool err = false;
@@ -369,9 +384,9 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
     const float kx = s.kx, ky = s.ky, kz = s.kz;
     float3 e1, e2;
     onb(kx, ky, kz, e1, e2);
-    float vx = upar * kx + up1 * e1.x + up2 * e2.x;   // scatterer velocity / v_th
-    float vy = upar * ky + up1 * e1.y + up2 * e2.y;
-    float vz = upar * kz + up1 * e1.z + up2 * e2.z;
+    float vx = __fmaf_rn(up2, e2.x, __fmaf_rn(upar, kx, up1 * e1.x));   // scatterer velocity / v_th
+    float vy = __fmaf_rn(up2, e2.y, __fmaf_rn(upar, ky, up1 * e1.y));
+    float vz = __fmaf_rn(up2, e2.z, __fmaf_rn(upar, kz, up1 * e1.z));
     int kind;
     if (ch > 0 || P.isotropic || L.phase != 0) kind = PH_ISO;
     else kind = fabsf(x_in - upar) < 0.2f ? PH_CORE : PH_WING;
@@ -405,7 +420,7 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
             }
         }
     }
-    float uout = ox * vx + oy * vy + oz * vz;
+    float uout = __fmaf_rn(oz, vz, __fmaf_rn(oy, vy, ox * vx));
     if (ch > 0) {
         double nu = __fma_rn(chnu, widen(uout * vthc), chnu);
         x_of_nu(P, s.cc, nu, s.xh, s.xl);
@@ -413,7 +428,7 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
         // nu_out = nu_in (1 + f)  <=>  x_out = x_in + (nu0/Delta nu + x_in) f
         float rec = (1.0f - mu) * recp;
         float f = __fdividef((uout - upar) * vthc - rec, 1.0f + rec);
-        pair_add(s.xh, s.xl, (s.cc.q0 + s.xh) * f);
+        pair_add(s.xh, s.xl, s.cc.q0 + s.xh, f);
     }
     if (!P.keep_dir) {
         s.kx = ox; s.ky = oy; s.kz = oz;
@@ -742,7 +757,7 @@ __global__ void __launch_bounds__(128, RG_PROP_MINB)
 k_propagate(const __grid_constant__ Params P, PacketsIn in, PacketsOut out, TraceOut tr) {
     Packet<NL> s;
     extern __shared__ uint32_t s_dyn[];
-    Tallies& tl = reinterpret_cast<Tallies*>(s_dyn + (kRing + 6 * NL) * blockDim.x)[threadIdx.x];
+    Tallies& tl = reinterpret_cast<Tallies*>(s_dyn + (kRing + 6 * NL) * kCols)[threadIdx.x];
     tl = Tallies{};
     const unsigned lane = threadIdx.x & 31u;
     bool have = false, drained = (int)lane >= P.lanes;
@@ -1411,7 +1426,7 @@ __global__ void k_sample_upar(Params P, long long n, const double* x, const floa
 // ---------------------------------------------------------------------------
 // draw rings, the u0 coefficient cache of each line, the event counters
 static size_t smem_bytes(int nline, int block) {
-    return (size_t)(kRing + nline * 6) * block * sizeof(float) + (size_t)block * sizeof(Tallies);
+    return (size_t)(kRing + nline * 6) * kCols * sizeof(float) + (size_t)block * sizeof(Tallies);
 }
 
 template <int NL>
@@ -1599,7 +1614,7 @@ cudaError_t launch_eval_voigt(long long n, const float* a, const double* x, floa
 cudaError_t launch_sample_upar(const Params& P, long long n, const double* x, const float* a, const uint64_t* id,
                                float* u, int32_t* nd, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_sample_upar<<<(unsigned)((n + 127) / 128), 128, kRing * 128 * sizeof(uint32_t), st>>>(P, n, x, a, id, u, nd);
+    k_sample_upar<<<(unsigned)((n + 127) / 128), 128, kRing * kCols * sizeof(uint32_t), st>>>(P, n, x, a, id, u, nd);
     return cudaGetLastError();
 }
 
