@@ -170,6 +170,7 @@ struct Params {
     int refill;
     // lanes of each warp that take packets (lanes_per_warp)
     int lanes;
+    unsigned wait;   // iterations that a lane may wait for company before a long piece of the loop
     // run scratch
     unsigned long long* counters;  // [CNT_N]
     unsigned long long* head;      // work-queue head

@@ -521,17 +521,18 @@ __device__ __forceinline__ void finish_packet(const Params& P, const Geo& G, con
 
 // Whether lanes that wait for a rare, long piece of the loop (an exact step, the
 // next packet) get it now: when they are a quarter of the lanes at work, when
-// nobody else is at work, or when they have waited four iterations.  Issued as
+// nobody else is at work, or when they have waited `wait` iterations.  Issued as
 // soon as one lane asks, a piece that one lane in fifty needs per iteration
 // goes out in every second iteration for one or two lanes.  The wait bounds
 // what a packet with a long history can lose.  Measured with the FP32 screen
 // below, sphere of tau0 = 1e6 (5e5 packets x 2000 scatterings): 126 ms issued
 // at once, 117 at an eighth, 107 at a quarter, 103 at a half or with longer
 // waits, which cost the batch of 200 models 6-20 % and short packets 5 %.
+// Where the packets do not fill the lanes the launch is as long as its longest
+// histories and nobody waits (wait = 1): batch of 45 600 packets 46.9 -> 42.9 ms.
 constexpr int kServeShare = 4;
-constexpr unsigned kServeWait = 4;
-__device__ __forceinline__ bool served(unsigned waiting, unsigned working, unsigned& held) {
-    if (working != 0u && kServeShare * __popc(waiting) < __popc(waiting | working) && ++held < kServeWait) return false;
+__device__ __forceinline__ bool served(unsigned waiting, unsigned working, unsigned& held, unsigned wait) {
+    if (working != 0u && kServeShare * __popc(waiting) < __popc(waiting | working) && ++held < wait) return false;
     held = 0u;
     return true;
 }
@@ -591,7 +592,7 @@ __device__ __forceinline__ void advance(const Params& P, const Geo& G, Packet<NL
     const unsigned waiting = __ballot_sync(kFull, need);
     if (waiting != 0u) {
         // lanes not served come back with the same step in the next iteration
-        if (!served(waiting, __ballot_sync(kFull, inter), held)) need = false;
+        if (!served(waiting, __ballot_sync(kFull, inter), held, P.wait)) need = false;
     }
     if (inter || need) {
         ++s.nsteps;
@@ -802,7 +803,7 @@ k_propagate(const __grid_constant__ Params P, PacketsIn in, PacketsOut out, Trac
         // results and take the next one together
         const bool ended = have && s.status != RASCAS_PK_ACTIVE_;
         unsigned m = __ballot_sync(kFull, ended || (!have && !drained));
-        if (m && served(m, __ballot_sync(kFull, have && !ended), idle)) {
+        if (m && served(m, __ballot_sync(kFull, have && !ended), idle, P.wait)) {
             if (ended) {
                 finish_packet<NL>(P, BATCH ? P.models[s.mi] : P.g, s, out, tl);
                 have = false;
@@ -1441,6 +1442,7 @@ static cudaError_t launch_nl(const Params& P_, const PacketsIn& in, const Packet
     // ms in full warps, 226 with 8 lanes, 212 with 4, 204 with 2, 205 with 1.
     // 40 000 packets fill half the warps' lanes: 637 ms, 670 spread over all.
     P.lanes = lanes_per_warp(in.n - in.first, (long long)grid * block / 64);
+    P.wait = in.n - in.first < (long long)grid * block ? 1u : 4u;
     // per-event traces are recorded by single-model runs without peeling only
     if (tr.nev && (P.nmodels > 0 || P.ndir > 0)) return cudaErrorInvalidValue;
     if (P.nmodels > 0) k_propagate<NL, false, true, false><<<grid, block, smem, st>>>(P, in, out, tr);
