@@ -206,10 +206,10 @@ RG_HD f2 f2_mul_f(f2 x, float y) {
     return fast_two_sum(p.h, fma_(x.l, y, p.l));
 }
 RG_HD f2 f2_neg(f2 x) { return {-x.h, -x.l}; }
-// split of a double (host or once per ray)
+// split of a double
 RG_HD f2 f2_of(double d) {
-    float h = (float)d;
-    return {h, (float)(d - (double)h)};
+    float h = narrow(d);
+    return {h, narrow(d - widen(h))};
 }
 RG_HD double f2_val(f2 x) { return (double)x.h + (double)x.l; }
 

@@ -253,27 +253,41 @@ __device__ __forceinline__ bool peel_step(const Params& P, Ray<NL>& r, bool grad
     return !linked_leaf(P.g, r.p, r.k, axis, r.w, lk, sl, nl);
 }
 
-// one peeling ray towards direction d (weight wt per sr, gas-frame frequency
-// nu_o_gas in the event's leaf), appended to the record buffer for the peel
-// kernel; one atomic per converged group of lanes.  A reservation at or past
-// the high-water mark asks the packet's warp to suspend.
+// Room in the record buffer for one event's peeling rays towards every
+// direction, for the converged group of lanes: one atomic for all of them (one
+// per direction put three returns of ~600 cycles into a scattering), the
+// rays of one direction next to each other (lane's first, then step per
+// direction).  A reservation at or past the high-water mark asks the packet's
+// warp to suspend.
+struct PeelSlots {
+    unsigned long long first;
+    unsigned step;
+};
 template <int NL>
-__device__ __forceinline__ void peel_emit(const Params& P, Packet<NL>& s, int d, float wt, double nu_o_gas,
-                                          Tallies& tl) {
+__device__ __forceinline__ PeelSlots peel_reserve(const Params& P, Packet<NL>& s, Tallies& tl) {
+    const unsigned m = __activemask();
+    const int lane = (int)(threadIdx.x & 31u), leader = __ffs(m) - 1;
+    const unsigned lanes = __popc(m);
+    unsigned long long base = 0;
+    if (lane == leader) base = atomicAdd(P.peel_count, (unsigned long long)(lanes * P.ndir));
+    base = __shfl_sync(m, base, leader);
+    if (base >= P.peel_hw) s.halt = true;
+    tl.peel_rays += P.ndir;
+    return {base + (unsigned long long)__popc(m & ((1u << lane) - 1u)), lanes};
+}
+
+// one peeling ray towards direction d (weight wt per sr, gas-frame frequency
+// nu_o_gas in the event's leaf) for the peel kernel
+template <int NL>
+__device__ __forceinline__ void peel_emit(const Params& P, const Packet<NL>& s, const PeelSlots& slots, int d, float wt,
+                                          double nu_o_gas) {
     double nu_ext = nu_o_gas;
     if (!at_rest(s.cc)) {
         const double b = __fma_rn(P.dirs[d][0], widen(s.cc.vx),
                                   __fma_rn(P.dirs[d][1], widen(s.cc.vy), P.dirs[d][2] * widen(s.cc.vz))) * (1.0 / kC);
         nu_ext = to_ext(nu_o_gas, b);
     }
-    const unsigned m = __activemask();
-    const int lane = (int)(threadIdx.x & 31u), leader = __ffs(m) - 1;
-    unsigned long long base = 0;
-    if (lane == leader) base = atomicAdd(P.peel_count, (unsigned long long)__popc(m));
-    base = __shfl_sync(m, base, leader);
-    const unsigned long long slot = base + (unsigned long long)__popc(m & ((1u << lane) - 1u));
-    if (base >= P.peel_hw) s.halt = true;
-    ++tl.peel_rays;
+    const unsigned long long slot = slots.first + (unsigned long long)(d * slots.step);
     if (slot >= P.peel_cap) return;   // cannot happen: peel_hw leaves room for every resident thread
     PeelRec& r = P.peel_rec[slot];
     r.p[0] = s.p0; r.p[1] = s.p1; r.p[2] = s.p2;
@@ -298,12 +312,13 @@ __device__ __forceinline__ void scatter_dust(const Params& P, Packet<NL>& s, Tal
     float mu = mu_sample(PH_HG, r_mu, P.dust_g, st);
     if (PEEL) {
         double nu_gas = nu_of_x(P, s.cc, s.xh, s.xl);   // coherent in the gas frame
+        const PeelSlots slots = peel_reserve<NL>(P, s, tl);
 #pragma unroll
         for (int d = 0; d < kMaxDirs; ++d) {
             if (d < P.ndir) {
                 float muo = s.kx * P.dir_kp[d][0][0] + s.ky * P.dir_kp[d][1][0] + s.kz * P.dir_kp[d][2][0];
                 float wt = phase_p(PH_HG, muo, P.dust_g) * (1.0f / kTwoPiF);
-                peel_emit<NL>(P, s, d, wt, nu_gas, tl);
+                peel_emit<NL>(P, s, slots, d, wt, nu_gas);
             }
         }
     }
@@ -401,6 +416,7 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
     const float recp = P.recoil ? L.recoil_pref * (P.line[0].nu0_f + s.xh * s.cc.dnu0_f) : 0.0f;
     if (PEEL) {
         double nu_in = nu_of_x(P, s.cc, s.xh, s.xl);
+        const PeelSlots slots = peel_reserve<NL>(P, s, tl);
 #pragma unroll
         for (int d = 0; d < kMaxDirs; ++d) {
             if (d < P.ndir) {
@@ -416,7 +432,7 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
                     nu_o = __fma_rn(nu_in, widen(f), nu_in);
                 }
                 float wt = phase_p(kind, muo, 0.0f) * (1.0f / kTwoPiF);
-                peel_emit<NL>(P, s, d, wt, nu_o, tl);
+                peel_emit<NL>(P, s, slots, d, wt, nu_o);
             }
         }
     }
@@ -564,10 +580,11 @@ __device__ __forceinline__ void advance(const Params& P, const Geo& G, Packet<NL
             s.enter = false;
             if (PEEL && s.fresh) {
                 // peeling of the isotropic emission (weight 1/4pi per sr)
+                const PeelSlots slots = peel_reserve<NL>(P, s, tl);
 #pragma unroll
                 for (int d = 0; d < kMaxDirs; ++d)
                     if (d < P.ndir)
-                        peel_emit<NL>(P, s, d, 1.0f / (2.0f * kTwoPiF), nu_gas, tl);
+                        peel_emit<NL>(P, s, slots, d, 1.0f / (2.0f * kTwoPiF), nu_gas);
             }
             s.fresh = false;
         }
@@ -1017,26 +1034,57 @@ __device__ __forceinline__ void ray_from_prep(const Params& P, unsigned long lon
     r.zero_run = 0;
 }
 
-// spectrum channel (or -1) and image pixel (or -1) of a peeled contribution
+// floor(t) for t known to within err, if that decides it
+__device__ __forceinline__ bool floor_certain(float t, float err, float& fl) {
+    fl = floorf(t);
+    return t - fl > err && (fl + 1.0f) - t > err;
+}
+
+// spectrum channel (or -1) and image pixel (or -1) of a peeled contribution:
+// the plain definitions' operations in FP64, unfused (exact ties bin as in the
+// oracle), where FP32 does not already decide the bin.  The plain form of a
+// record takes some 70 FP64 instructions, three divisions among them; all but
+// about one record in a thousand end with four subtractions.  With the merged
+// reservation, outflow of 30000 packets (1.6e8 rays): 204 -> 176 ms, the prep
+// pass 25.9 -> 11.5 ms of it.
 __device__ __forceinline__ void peel_bins(const Params& P, const PeelRec& q, int& ch, long long& px) {
     const int nbin = P.g.nbin;
-    // the plain definitions' operations, unfused (exact ties bin as in the oracle)
-    const double t = __ddiv_rn(__dsub_rn(q.nu_ext, P.g.nu_lo), P.g.nu_range);
-    const double fb = floor(__dmul_rn(t, (double)nbin));
-    ch = (fb >= 0.0 && fb < (double)nbin) ? (int)fb : -1;
+    const double dn = __dsub_rn(q.nu_ext, P.g.nu_lo);
+    float fl;
+    // quotient, product and both roundings to FP32: 4e-7 of the value
+    const float tb = narrow(dn) * __fdividef((float)nbin, narrow(P.g.nu_range));
+    if (floor_certain(tb, 1e-6f * (fabsf(tb) + 1.0f), fl)) {
+        ch = (fl >= 0.0f && fl < (float)nbin) ? (int)fl : -1;
+    } else {
+        const double fb = floor(__dmul_rn(__ddiv_rn(dn, P.g.nu_range), (double)nbin));
+        ch = (fb >= 0.0 && fb < (double)nbin) ? (int)fb : -1;
+    }
     px = -1;
     if (P.npix > 0) {
         const int d = q.d;
         const double r0 = __dsub_rn(q.p[0], P.img_c[0]), r1 = __dsub_rn(q.p[1], P.img_c[1]);
         const double r2 = __dsub_rn(q.p[2], P.img_c[2]);
-        const double u = __dadd_rn(__dadd_rn(__dmul_rn(r0, P.eu[d][0]), __dmul_rn(r1, P.eu[d][1])),
-                                   __dmul_rn(r2, P.eu[d][2]));
-        const double v = __dadd_rn(__dadd_rn(__dmul_rn(r0, P.ev[d][0]), __dmul_rn(r1, P.ev[d][1])),
-                                   __dmul_rn(r2, P.ev[d][2]));
-        const double fu = floor(__dmul_rn(__dadd_rn(__ddiv_rn(u, P.fov), 0.5), (double)P.npix));
-        const double fv = floor(__dmul_rn(__dadd_rn(__ddiv_rn(v, P.fov), 0.5), (double)P.npix));
-        if (fu >= 0.0 && fu < (double)P.npix && fv >= 0.0 && fv < (double)P.npix)
-            px = (long long)fv * P.npix + (long long)fu;
+        const float a0 = narrow(r0), a1 = narrow(r1), a2 = narrow(r2), np = (float)P.npix;
+        const float per = __fdividef(np, narrow(P.fov));
+        const float uf = (a0 * narrow(P.eu[d][0]) + a1 * narrow(P.eu[d][1]) + a2 * narrow(P.eu[d][2])) * per + 0.5f * np;
+        const float vf = (a0 * narrow(P.ev[d][0]) + a1 * narrow(P.ev[d][1]) + a2 * narrow(P.ev[d][2])) * per + 0.5f * np;
+        // each of the three terms carries 2e-7 of itself, the sum and the
+        // product with `per` as much again; e has entries of at most 2
+        const float err = 2e-6f * ((fabsf(a0) + fabsf(a1) + fabsf(a2)) * per + np);
+        float fu, fv;
+        const bool cu = floor_certain(uf, err, fu), cv = floor_certain(vf, err, fv);
+        if (cu && cv) {
+            if (fu >= 0.0f && fu < np && fv >= 0.0f && fv < np) px = (long long)(int)fv * P.npix + (long long)(int)fu;
+        } else {
+            const double u = __dadd_rn(__dadd_rn(__dmul_rn(r0, P.eu[d][0]), __dmul_rn(r1, P.eu[d][1])),
+                                       __dmul_rn(r2, P.eu[d][2]));
+            const double v = __dadd_rn(__dadd_rn(__dmul_rn(r0, P.ev[d][0]), __dmul_rn(r1, P.ev[d][1])),
+                                       __dmul_rn(r2, P.ev[d][2]));
+            const double gu = floor(__dmul_rn(__dadd_rn(__ddiv_rn(u, P.fov), 0.5), (double)P.npix));
+            const double gv = floor(__dmul_rn(__dadd_rn(__ddiv_rn(v, P.fov), 0.5), (double)P.npix));
+            if (gu >= 0.0 && gu < (double)P.npix && gv >= 0.0 && gv < (double)P.npix)
+                px = (long long)gv * P.npix + (long long)gu;
+        }
     }
 }
 
@@ -1050,7 +1098,7 @@ __device__ __forceinline__ bool first_leaf_dark(const Params& P, const Ray<NL>& 
     f2 beta;
     const float kap = ray_opacity<NL>(P, r.R, r0, r1, kl, xh, xl, beta);
     int axis;
-    const double tf = face_distance(r.p, r.k, r.inv, r.w, axis);
+    const double tf = exit_distance(r.p, r.k, r.inv, r.w, axis);
     bool border = false;
     double l = tf;
     if (__float_as_int(r1.w) & kFlagBorder) {
@@ -1130,8 +1178,10 @@ __global__ void __launch_bounds__(256) k_peel_prep(const Params* __restrict__ G)
     flush(P, dark_cells, CNT_LEAF_LOADS);
 }
 
+// Five blocks per SM (96 registers) for the forward walk: galaxy, 2^16 packets,
+// 47.2 -> 43.1 ms against four (six: 43.6); the adjoint's registers allow three.
 template <int NL, bool ADJ>
-__global__ void __launch_bounds__(128, ADJ ? 3 : 4) k_peel(const Params* __restrict__ G) {
+__global__ void __launch_bounds__(128, ADJ ? 3 : 5) k_peel(const Params* __restrict__ G) {
     const Params& P = *G;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned long long n = *P.peel_nlive;   // the rays the prep pass listed
