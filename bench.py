@@ -35,20 +35,22 @@ METRIC = "scatterings/sec & packets/sec on 1 GB300 vs oracle; batched vs plain s
 WORKLOAD = ("static H I + dust sphere: 8^3 root refined to 64^3-equivalent octree (172992 leaves), "
             "tau0=1e6 centre-to-edge, T=1e4 K, tau_dust=1, albedo 0.32, packets from the centre at x=0")
 # Instruction counts of k_propagate per scattering on this workload, from one
-# ncu capture of the kernel (an uncapped launch of 65536 packets of the same
+# ncu capture of the kernel (an uncapped launch of 524288 packets of the same
 # sphere; smsp__inst_executed.sum and smsp__inst_executed_pipe_*.sum divided
 # by the launch's scatterings), and the active lanes per warp instruction of
 # the same capture.  They are constants of the code and the workload, so the
 # bench multiplies them by its own live scattering rate.
-INST_PER_SCATT = 6044032067435 / 111923728554
-LANES_PER_INST = 106529112851470 / 6044032067435
+INST_PER_SCATT = 5639892421749 / 111923728554
+LANES_PER_INST = 107366308850329 / 5639892421749
 # pipe -> warp instructions per scattering of the same capture (FP32 FMA,
 # FP64, special-function unit)
-PIPE_PER_SCATT = {"fma": 2877856853460 / 111923728554, "fp64": 83386945512 / 111923728554,
-                  "xu": 166026282325 / 111923728554}
+PIPE_PER_SCATT = {"fma": 2821713684031 / 111923728554, "fp64": 59794947584 / 111923728554,
+                  "xu": 169162376323 / 111923728554}
 # DRAM bytes per leaf visit of k_ray_tau on the synthetic galaxy
 # (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of 2^18
-# rays from emitting leaves, 59 732 805 leaf visits)
+# rays from emitting leaves, 59 732 805 leaf visits, with the neighbour search
+# by records; the walk by face links moved 46.6 bytes per visit through a
+# galaxy of 3.2e6 leaves)
 RAY_DRAM_BYTES_PER_VISIT = (4.107982e9 + 49.11232e6) / 59732805
 
 
