@@ -220,7 +220,8 @@ int rascas_set_stream(rascas_ctx *ctx, void *stream);
 /* Copy an octree and its leaf fields to the device (mem: where the arrays
  * live).  Validates the tree (RASCAS_E_ARG on malformed input), derives the
  * father and neighbour links of Sect. 4.3 and the leaf levels, and packs the
- * fields into 32-byte leaf records. */
+ * fields into 32-byte leaf records; a second 32 bytes per leaf hold the cells
+ * across its faces, which the ray walks follow. */
 int rascas_load_octree(rascas_ctx *ctx, const rascas_octree *tree, int mem);
 /* The computational domain of Sect. 4 (sphere, shell, slab periodic in x and
  * y, cube) inside the unit box.  Leaves that cannot reach its border are

@@ -121,20 +121,6 @@ struct Ray {
     int n, zero_run;
 };
 
-template <int NL>
-__device__ __forceinline__ void ray_start(const Params& P, Ray<NL>& r, double p0, double p1, double p2, Where w,
-                                          double k0, double k1, double k2, double nu_ext) {
-    r.p[0] = p0; r.p[1] = p1; r.p[2] = p2;
-    r.k[0] = k0; r.k[1] = k1; r.k[2] = k2;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) r.inv[j] = is_zero(r.k[j]) ? 0.0 : __drcp_rn(r.k[j]);
-    r.w = w;
-    ray_nu<NL>(P, nu_ext, r.k, r.R);
-    r.tau = f2{0.0f, 0.0f};
-    r.n = 0;
-    r.zero_run = 0;
-}
-
 // one leaf of the walk; true when the ray is done (border, box edge, tau
 // beyond tstop, or a stuck walk)
 template <int NL>
