@@ -206,7 +206,8 @@ int rascas_create(rascas_ctx **out, int device);
 int rascas_destroy(rascas_ctx *ctx);
 /* Text of the last error on this context (never NULL). */
 const char *rascas_last_error(const rascas_ctx *ctx);
-/* Stream for all later work (a cudaStream_t passed as void*, NULL = legacy). */
+/* Stream for all later work, uploads of the set-up calls included (a
+ * cudaStream_t passed as void*, NULL = legacy); it has to outlive its use here. */
 int rascas_set_stream(rascas_ctx *ctx, void *stream);
 
 /* ---- problem set-up (the paper's problem statement: mesh + fields,

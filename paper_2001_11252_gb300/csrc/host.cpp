@@ -123,6 +123,16 @@ cudaError_t to_host(void* dst, const void* src, size_t bytes, int mem) {
     return cudaSuccess;
 }
 
+// host data to the device, there when the call returns: queued on the context's
+// stream, behind the work in flight there that may still read the old data, and
+// waited for.  A cudaMemcpy from pageable memory may return before its last
+// bytes have arrived, and orders nothing with a non-blocking stream.
+cudaError_t upload(const rascas_ctx* ctx, void* dst, const void* src, size_t bytes) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, ctx->stream);
+    const cudaError_t w = cudaStreamSynchronize(ctx->stream);
+    return e != cudaSuccess ? e : w;
+}
+
 // leaf flags for a domain: a leaf is interior when it lies strictly inside the
 // domain with a relative margin; then no ray from inside it reaches the border
 // before one of its faces, and the walk skips the border distance there
@@ -373,10 +383,10 @@ int rascas_load_octree(rascas_ctx* ctx, const rascas_octree* t, int mem) {
     CK(ctx->d_nbr.ensure(M.nbr.size() * 4));
     CK(ctx->d_top.ensure(M.top.size() * 4));
     CK(ctx->d_link.ensure(M.rec.size() * 4));
-    CK(cudaMemcpy(ctx->d_rec.p, M.rec.data(), M.rec.size() * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(ctx->d_son.p, M.son.data(), M.son.size() * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(ctx->d_nbr.p, M.nbr.data(), M.nbr.size() * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(ctx->d_top.p, M.top.data(), M.top.size() * 4, cudaMemcpyHostToDevice));
+    CK(upload(ctx, ctx->d_rec.p, M.rec.data(), M.rec.size() * 4));
+    CK(upload(ctx, ctx->d_son.p, M.son.data(), M.son.size() * 4));
+    CK(upload(ctx, ctx->d_nbr.p, M.nbr.data(), M.nbr.size() * 4));
+    CK(upload(ctx, ctx->d_top.p, M.top.data(), M.top.size() * 4));
     Params& P = ctx->P;
     P.g.rec = (const float4*)ctx->d_rec.p;
     P.g.son = (const int*)ctx->d_son.p;
@@ -412,7 +422,7 @@ int rascas_set_domain(rascas_ctx* ctx, const rascas_domain* d) {
     if (ctx->has_mesh) {
         CK(cudaSetDevice(ctx->device));
         mesh_flags(ctx->mesh, &ctx->dom);
-        CK(cudaMemcpy(ctx->d_rec.p, ctx->mesh.rec.data(), ctx->mesh.rec.size() * 4, cudaMemcpyHostToDevice));
+        CK(upload(ctx, ctx->d_rec.p, ctx->mesh.rec.data(), ctx->mesh.rec.size() * 4));
     }
     return RASCAS_OK;
 }
@@ -1161,6 +1171,9 @@ int rascas_load_batch(rascas_ctx* ctx, const rascas_model* models, int32_t nmode
     }
     CK(cudaMemcpy(B.d_geo.p, geo.data(), sizeof(rg::Geo) * nmodels, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(B.d_first.p, B.first.data(), sizeof(long long) * (nmodels + 1), cudaMemcpyHostToDevice));
+    // the copies above are on the legacy stream and may still be under way (see
+    // upload); the runs take a non-blocking one
+    CK(cudaStreamSynchronize(cudaStreamLegacy));
     B.nmodels = nmodels;
     B.nbin = nbin;
     B.npackets = npk;
@@ -1432,7 +1445,7 @@ int rascas_update_fields(rascas_ctx* ctx, const float* n_HI, const float* vx, co
         const float* src[7] = {n_HI, vx, vy, vz, T, n_dust, n_metal};
         for (size_t i = 0; i < N; ++i)
             for (int j = 0; j < 7; ++j) ctx->mesh.rec[8 * i + j] = src[j] ? src[j][i] : 0.0f;
-        CK(cudaMemcpy(ctx->d_rec.p, ctx->mesh.rec.data(), N * 32, cudaMemcpyHostToDevice));
+        CK(upload(ctx, ctx->d_rec.p, ctx->mesh.rec.data(), N * 32));
     }
     if (n_metal) ctx->mesh.has_metal = true;
     return RASCAS_OK;
