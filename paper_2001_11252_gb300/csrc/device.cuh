@@ -168,35 +168,31 @@ struct Rng {
 // formed in FP64 and its rounding to FP32 is fed back into exp(-x^2) to first
 // order, so H keeps ~1e-7 relative accuracy where exp(-x^2) dominates.
 // ---------------------------------------------------------------------------
+// Roundings are written out where a multiply-add could form or not, in both
+// forms of H: a packet's history depends on them, which must not change with
+// the code around.
+// the damping wing q of H = sqrt(pi) q + exp(-x^2), 0 in the core
+__device__ __forceinline__ float wing_q(float a, float x2) {
+    const float z = __fdividef(x2 - 0.855f, x2 + 3.42f);
+    if (!(z > 0.0f)) return 0.0f;
+    const float pz = __fmaf_rn(z, __fmaf_rn(z, __fmaf_rn(5.674f, z, -9.207f), 4.421f), 0.1117f);
+    return z * (1.0f + __fdividef(21.0f, x2)) * __fdividef(a, kPiF * (x2 + 1.0f)) * pz;
+}
+
 __device__ __forceinline__ float voigt_h(float a, double x) {
-    double x2d = x * x;
-    float x2 = narrow(x2d);
-    float lo = narrow(x2d - widen(x2));
-    float e = expf(-x2) * (1.0f - lo);
-    float z = __fdividef(x2 - 0.855f, x2 + 3.42f);
-    float q = 0.0f;
-    if (z > 0.0f) {
-        q = z * (1.0f + __fdividef(21.0f, x2)) * __fdividef(a, kPiF * (x2 + 1.0f)) *
-            (0.1117f + z * (4.421f + z * (-9.207f + 5.674f * z)));
-    }
-    return kSqrtPiF * q + e;
+    const double x2d = __dmul_rn(x, x);
+    const float x2 = narrow(x2d);
+    const float lo = narrow(__dsub_rn(x2d, widen(x2)));
+    return __fmaf_rn(expf(-x2), 1.0f - lo, __fmul_rn(kSqrtPiF, wing_q(a, x2)));
 }
 
 // Same function for x carried as an unevaluated FP32 pair x = xh + xl: x^2 is
 // xh^2 plus its exact rounding error plus 2 xh xl, all in FP32.
 __device__ __forceinline__ float voigt_h2(float a, float xh, float xl) {
-    // roundings written out where a multiply-add could form or not: a packet's
-    // history depends on them, which must not change with the code around
-    float x2 = __fmul_rn(xh, xh);
-    float lo = fmaf(xh, xh, -x2) + 2.0f * xh * xl;
-    float e = expf(-x2) * (1.0f - lo);
-    float z = __fdividef(x2 - 0.855f, x2 + 3.42f);
-    float q = 0.0f;
-    if (z > 0.0f) {
-        q = z * (1.0f + __fdividef(21.0f, x2)) * __fdividef(a, kPiF * (x2 + 1.0f)) *
-            (0.1117f + z * (4.421f + z * (-9.207f + 5.674f * z)));
-    }
-    return __fadd_rn(__fmul_rn(kSqrtPiF, q), e);
+    const float x2 = __fmul_rn(xh, xh);
+    const float lo = __fmaf_rn(2.0f * xh, xl, fmaf(xh, xh, -x2));
+    const float e = __fmul_rn(expf(-x2), 1.0f - lo);
+    return __fadd_rn(__fmul_rn(kSqrtPiF, wing_q(a, x2)), e);
 }
 
 // H with its partial derivatives in a and x (the derivative of this
@@ -222,14 +218,16 @@ __device__ __forceinline__ void voigt_derivs(float a, float x, float& H, float& 
 }
 
 // H by the option the kernels are built for (kFaddeeva), x as an FP32 pair
+template <int NL>
 __device__ __forceinline__ float voigt_sel(float a, float xh, float xl) {
-    if constexpr (kFaddeeva) return faddeeva_h(a, xh, xl);
+    if constexpr (kFaddeeva) return faddeeva_h<(NL > 2)>(a, xh, xl);
     else return voigt_h2(a, xh, xl);
 }
+template <int NL>
 __device__ __forceinline__ float voigt_sel(float a, double x) {
     if constexpr (kFaddeeva) {
         const float xh = narrow(x);
-        return faddeeva_h(a, xh, narrow(x - widen(xh)));
+        return faddeeva_h<(NL > 2)>(a, xh, narrow(x - widen(xh)));
     } else {
         return voigt_h(a, x);
     }
@@ -833,9 +831,10 @@ __device__ __forceinline__ double nu_of_x(const Params& P, const CellCache<NL>& 
 }
 template <int NL>
 __device__ __forceinline__ void x_of_nu(const Params& P, const CellCache<NL>& cc, double nu, float& xh, float& xl) {
-    double x = (nu - P.line[0].nu0) * cc.invdnu[0];
+    // no multiply-add across the two roundings: packets' frequencies depend on it
+    const double x = __dmul_rn(nu - P.line[0].nu0, cc.invdnu[0]);
     xh = narrow(x);
-    xl = narrow(x - widen(xh));
+    xl = narrow(__dsub_rn(x, widen(xh)));
 }
 
 // total opacity (cm^-1) at the line-0 Doppler offset x = xh + xl; cum[i] = the
@@ -845,13 +844,13 @@ __device__ __forceinline__ void x_of_nu(const Params& P, const CellCache<NL>& cc
 template <int NL>
 __device__ __forceinline__ float opacity_x(const Params& P, const CellCache<NL>& cc, float xh, float xl,
                                            float cum[NL], float xin[NL]) {
-    cum[0] = __fmaf_rn(cc.kap0[0], voigt_sel(cc.a[0], xh, xl), cc.kap_d);
+    cum[0] = __fmaf_rn(cc.kap0[0], voigt_sel<NL>(cc.a[0], xh, xl), cc.kap_d);
     xin[0] = xh;
 #pragma unroll
     for (int i = 1; i < NL; ++i) {
         double x = __fma_rn(widen(xh) + widen(xl), cc.xb[i], cc.xa[i]);
         xin[i] = narrow(x);
-        cum[i] = __fmaf_rn(cc.kap0[i], voigt_sel(cc.a[i], x), cum[i - 1]);
+        cum[i] = __fmaf_rn(cc.kap0[i], voigt_sel<NL>(cc.a[i], x), cum[i - 1]);
     }
     return cum[NL - 1];
 }
@@ -935,7 +934,7 @@ __device__ __forceinline__ float ray_opacity(const Params& P, const RayNu<NL>& R
         const float n = (L.dens == 1 ? r1.z : r0.x) * L.abund;
         xh[i] = x.h;
         xl[i] = x.l;
-        kl[i] = n * L.sig_pref * rs * voigt_sel(L.a_pref * rs, x.h, x.l);
+        kl[i] = n * L.sig_pref * rs * voigt_sel<NL>(L.a_pref * rs, x.h, x.l);
         tot += kl[i];
     }
     return tot;

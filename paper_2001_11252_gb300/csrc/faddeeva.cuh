@@ -36,6 +36,27 @@ RG_HD void sincospi_f(float x, float* s, float* c) {
     *c = (float)std::cos(t);
 #endif
 }
+// Products and sums with their roundings written out: a packet's history
+// depends on them, and a compiler that may choose which product of a sum of two
+// to fuse chose differently from one kernel to the next (with two lines, the
+// peeling kernel and the plain one gave different histories).  dot2 = a b + c d
+// and det2 = a b - c d round the second product, then take one multiply-add.
+RG_HD float mul_(float a, float b) {
+#if defined(__CUDA_ARCH__)
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+RG_HD float add_(float a, float b) {
+#if defined(__CUDA_ARCH__)
+    return __fadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+RG_HD float dot2(float a, float b, float c, float d) { return fma_(a, b, mul_(c, d)); }
+RG_HD float det2(float a, float b, float c, float d) { return fma_(a, b, -mul_(c, d)); }
 RG_HD float sinpi_f(float x) {
 #if defined(__CUDA_ARCH__)
     return sinpif(x);
@@ -103,20 +124,23 @@ RG_HD void fad_nodes(float a, float xh, float xl, int m, float& H, float& K, std
 RG_HD void fad_far(float a, float x, float& H, float& K) {
     const float q = fdiv_fast(1.0f, fmaf(x, x, a * a));
     const float ur = x * q, ui = -a * q;
-    const float vr = ur * ur - ui * ui, vi = 2.0f * ur * ui;
+    const float vr = det2(ur, ur, ui, ui), vi = 2.0f * ur * ui;
     float pr = 945.0f / 32.0f, pi = 0.0f;
     const float c[5] = {105.0f / 16.0f, 15.0f / 8.0f, 0.75f, 0.5f, 1.0f};
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        const float tr = pr * vr - pi * vi;
-        pi = pr * vi + pi * vr;
+        const float tr = det2(pr, vr, pi, vi);
+        pi = dot2(pr, vi, pi, vr);
         pr = tr + c[k];
     }
-    H = -(ur * pi + ui * pr) * (1.0f / kFadSqrtPiF);
-    K = (ur * pr - ui * pi) * (1.0f / kFadSqrtPiF);
+    H = -dot2(ui, pr, ur, pi) * (1.0f / kFadSqrtPiF);
+    K = det2(ur, pr, ui, pi) * (1.0f / kFadSqrtPiF);
 }
 
-// H and K = Im w at z = (xh + xl) + i a, x carried as an FP32 pair
+// H and K = Im w at z = (xh + xl) + i a, x carried as an FP32 pair.  kFused:
+// |v|^2 and Re v^2 by multiply-adds or by rounded products; seeded histories
+// have had the former with three and four lines, the latter with one and two.
+template <bool kFused = false>
 RG_HD void faddeeva_hk(float a, float xh, float xl, float& H, float& K) {
     if (!(fabsf(xh) <= 8.0f)) {
         fad_far(a, xh + xl, H, K);
@@ -132,7 +156,8 @@ RG_HD void faddeeva_hk(float a, float xh, float xl, float& H, float& K) {
     const float pr = d + mf;
     const float ur = fmaf(a, a, -d * pr), ui = -a * (2.0f * d + mf);
     float er, ei;
-    if (ur * ur + ui * ui < 0.25f) {
+    const float u2 = dot2(ur, ur, ui, ui);
+    if (u2 < 0.25f) {
         // E(u) = sum_k u^k / (k + 1)!
         er = 1.0f / 362880.0f;
         ei = 0.0f;
@@ -140,8 +165,8 @@ RG_HD void faddeeva_hk(float a, float xh, float xl, float& H, float& K) {
                             1.0f / 24.0f, 1.0f / 6.0f, 0.5f, 1.0f};
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const float tr = er * ur - ei * ui;
-            ei = er * ui + ei * ur;
+            const float tr = det2(er, ur, ei, ui);
+            ei = dot2(er, ui, ei, ur);
             er = tr + c[k];
         }
     } else {
@@ -149,37 +174,39 @@ RG_HD void faddeeva_hk(float a, float xh, float xl, float& H, float& K) {
         float su, cu;
         sincosf(ui, &su, &cu);
         const float sh = sinf(0.5f * ui);
-        const float nr = expm1f(ur) * cu - 2.0f * sh * sh, ni = expf(ur) * su;
-        const float q = fdiv_fast(1.0f, ur * ur + ui * ui);
-        er = (nr * ur + ni * ui) * q;
-        ei = (ni * ur - nr * ui) * q;
+        const float nr = det2(expm1f(ur), cu, 2.0f * sh, sh), ni = expf(ur) * su;
+        const float q = fdiv_fast(1.0f, u2);
+        er = dot2(ni, ui, nr, ur) * q;
+        ei = det2(ni, ur, nr, ui) * q;
     }
     const float cm = (0.5f / kFadPiF) * expf(-0.25f * mf * mf);
-    H = fmaf(-cm, er * a + ei * pr, H);
-    K = fmaf(cm, er * pr - ei * a, K);
+    H = fmaf(-cm, dot2(er, a, ei, pr), H);
+    K = fmaf(cm, det2(er, pr, ei, a), K);
     // residue part: 2 e^{-z^2} B(v), e^{-z^2} = e^{a^2 - x^2} (cos 2ax - i sin 2ax)
-    const float x2 = xh * xh;
-    const float lo = fmaf(xh, xh, -x2) + 2.0f * xh * xl;
+    const float x2 = mul_(xh, xh);
+    const float lo = fma_(2.0f * xh, xl, fmaf(xh, xh, -x2));
     const float g = expf(fmaf(a, a, -x2)) * (1.0f - lo);
     float s2, c2;
     sincosf(2.0f * a * xh, &s2, &c2);
     const float gr = g * c2, gi = -g * s2;
     const float vr = -4.0f * kFadPiF * a, vi = 4.0f * kFadPiF * d;
     float br, bi;
-    if (vr * vr + vi * vi < 1.0f) {
+    const float vr2 = mul_(vr, vr), vi2 = mul_(vi, vi);
+    const float v2 = kFused ? fma_(vr, vr, vi2) : add_(vr2, vi2);
+    if (v2 < 1.0f) {
         // B(v) = 1/2 + v/12 - v^3/720 + v^5/30240 - v^7/1209600 + v^9/47900160
-        const float wr = vr * vr - vi * vi, wi = 2.0f * vr * vi;
+        const float wr = kFused ? fma_(vr, vr, -vi2) : add_(vr2, -vi2), wi = 2.0f * vr * vi;
         br = 1.0f / 47900160.0f;
         bi = 0.0f;
         const float c[4] = {-1.0f / 1209600.0f, 1.0f / 30240.0f, -1.0f / 720.0f, 1.0f / 12.0f};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float tr = br * wr - bi * wi;
-            bi = br * wi + bi * wr;
+            const float tr = det2(br, wr, bi, wi);
+            bi = dot2(br, wi, bi, wr);
             br = tr + c[k];
         }
-        const float tr = br * vr - bi * vi;
-        bi = br * vi + bi * vr;
+        const float tr = det2(br, vr, bi, vi);
+        bi = dot2(br, vi, bi, vr);
         br = tr + 0.5f;
     } else {
         // 1 - e^{-v} = (2 sin^2(2 pi d) - expm1(4 pi a) cos(4 pi d)) + i e^{4 pi a} sin(4 pi d)
@@ -187,18 +214,19 @@ RG_HD void faddeeva_hk(float a, float xh, float xl, float& H, float& K) {
         sincospi_f(4.0f * d, &s4, &c4);
         const float sd = sinpi_f(2.0f * d);
         const float ea = 4.0f * kFadPiF * a;
-        const float Dr = 2.0f * sd * sd - expm1f(ea) * c4, Di = expf(ea) * s4;
-        const float qd = fdiv_fast(1.0f, Dr * Dr + Di * Di), qv = fdiv_fast(1.0f, vr * vr + vi * vi);
-        br = Dr * qd - vr * qv;
-        bi = vi * qv - Di * qd;
+        const float Dr = det2(2.0f * sd, sd, expm1f(ea), c4), Di = expf(ea) * s4;
+        const float qd = fdiv_fast(1.0f, dot2(Di, Di, Dr, Dr)), qv = fdiv_fast(1.0f, v2);
+        br = det2(Dr, qd, vr, qv);
+        bi = det2(vi, qv, Di, qd);
     }
-    H = fmaf(2.0f, gr * br - gi * bi, H);
-    K = fmaf(2.0f, gr * bi + gi * br, K);
+    H = fmaf(2.0f, det2(gr, br, gi, bi), H);
+    K = fmaf(2.0f, dot2(gr, bi, gi, br), K);
 }
 
+template <bool kFused = false>
 RG_HD float faddeeva_h(float a, float xh, float xl) {
     float H, K;
-    faddeeva_hk(a, xh, xl, H, K);
+    faddeeva_hk<kFused>(a, xh, xl, H, K);
     return H;
 }
 
@@ -210,22 +238,22 @@ RG_HD void faddeeva_derivs(float a, float x, float& H, float& Ha, float& Hx) {
     float K;
     faddeeva_hk(a, x, 0.0f, H, K);
     if (fabsf(x) <= 8.0f) {
-        Hx = 2.0f * (a * K - x * H);
-        Ha = 2.0f * (x * K + a * H) - 2.0f / kFadSqrtPiF;
+        Hx = 2.0f * det2(a, K, x, H);
+        Ha = 2.0f * dot2(x, K, a, H) - 2.0f / kFadSqrtPiF;
         return;
     }
     const float q = fdiv_fast(1.0f, fmaf(x, x, a * a));
     const float ur = x * q, ui = -a * q;
-    const float vr = ur * ur - ui * ui, vi = 2.0f * ur * ui;
+    const float vr = det2(ur, ur, ui, ui), vi = 2.0f * ur * ui;
     float pr = 10395.0f / 32.0f, pi = 0.0f;
     const float c[5] = {945.0f / 16.0f, 105.0f / 8.0f, 15.0f / 4.0f, 1.5f, 1.0f};
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        const float tr = pr * vr - pi * vi;
-        pi = pr * vi + pi * vr;
+        const float tr = det2(pr, vr, pi, vi);
+        pi = dot2(pr, vi, pi, vr);
         pr = tr + c[k];
     }
-    const float tr = vr * pr - vi * pi, ti = vr * pi + vi * pr;
+    const float tr = det2(vr, pr, vi, pi), ti = dot2(vr, pi, vi, pr);
     Hx = ti * (1.0f / kFadSqrtPiF);
     Ha = tr * (1.0f / kFadSqrtPiF);
 }

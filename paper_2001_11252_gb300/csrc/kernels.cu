@@ -428,8 +428,8 @@ __device__ __forceinline__ void scatter_line(const Params& P, const Geo& G, Pack
         x_of_nu(P, s.cc, nu, s.xh, s.xl);
     } else {
         // nu_out = nu_in (1 + f)  <=>  x_out = x_in + (nu0/Delta nu + x_in) f
-        float rec = (1.0f - mu) * recp;
-        float f = __fdividef((uout - upar) * vthc - rec, 1.0f + rec);
+        const float rec = __fmul_rn(1.0f - mu, recp);
+        const float f = __fdividef(__fmaf_rn(uout - upar, vthc, -rec), __fadd_rn(1.0f, rec));
         pair_add(s.xh, s.xl, s.cc.q0 + s.xh, f);
     }
     if (!P.keep_dir) {
