@@ -793,8 +793,15 @@ k_propagate(const __grid_constant__ Params P, PacketsIn in, PacketsOut out, Trac
         }
         if (PEEL && __any_sync(kFull, have && s.halt)) {
             // the record buffer is nearly full: park this warp's packets for
-            // the next round, after the peel kernel has drained the records
+            // the next round, after the peel kernel has drained the records.
+            // There is no next round where another warp reaches a limit, so
+            // packets that have ended are written now, the others as in flight.
+            if (have && s.status != RASCAS_PK_ACTIVE_) {
+                finish_packet<NL>(P, P.g, s, out, tl);
+                have = false;
+            }
             if (have) {
+                if (P.limits && out.status) out.status[s.idx] = RASCAS_PK_ACTIVE_;
                 s.halt = false;
                 static_cast<Packet<NL>*>(P.save)[gt] = s;
                 P.save_flag[gt] = 1;
