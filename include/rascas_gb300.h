@@ -241,10 +241,11 @@ int rascas_set_lines(rascas_ctx *ctx, const rascas_line *lines, int32_t nline, c
 int rascas_set_physics(rascas_ctx *ctx, const rascas_physics *phys);
 /* Bounded device work.  The persistent kernels of rascas_propagate, _trace,
  * _propagate_noalloc and _propagate_batch, and the peeling kernel, give up
- * once a thread has run max_iterations loop iterations (at most one walk step
- * per iteration; 0 = no limit, at most 2^32 - 1) or a launch has run
- * time_limit_s seconds of the GPU's global timer (0 = no limit; checked
- * every 256 iterations).  The call then returns RASCAS_E_TIMEOUT; packets in
+ * once a thread has done max_iterations walk steps and has more to do (0 = no
+ * limit, at most 2^32 - 1; a packet counts for at least one step; threads that
+ * wait for others, three loop iterations at most before a step or a packet, spend
+ * nothing) or a launch has run time_limit_s seconds of the GPU's global timer
+ * (0 = no limit; checked every 256 loop iterations).  The call then returns RASCAS_E_TIMEOUT; packets in
  * flight are left unfinished (status RASCAS_PK_ACTIVE where statuses are
  * returned), packets never started keep their output slots untouched, and
  * tallies hold what was accumulated.  The context stays usable.  Default:

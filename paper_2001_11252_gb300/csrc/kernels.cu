@@ -44,7 +44,7 @@ struct Tallies {
     uint32_t cross, peel_rays, peel_cells, trials, leaf_loads, son_loads, nbor_loads;
     uint32_t scatt_line, scatt_dust;
     uint32_t pk, esc, abs, cap, err;
-    uint32_t pad;
+    uint32_t spent;   // walk steps of this launch by the packets that have ended (one at least for each)
 };
 static_assert(sizeof(Tallies) == 15 * 4, "odd word stride");
 
@@ -509,6 +509,7 @@ __device__ __forceinline__ void finish_packet(const Params& P, const Geo& G, con
     if (out.path) out.path[i] = s.path;
     if (out.pos) { out.pos[3 * i] = s.p0; out.pos[3 * i + 1] = s.p1; out.pos[3 * i + 2] = s.p2; }
     if (out.dir) { out.dir[3 * i] = s.kd0; out.dir[3 * i + 1] = s.kd1; out.dir[3 * i + 2] = s.kd2; }
+    tl.spent += s.nsteps > 0 ? (uint32_t)s.nsteps : 1u;
     ++tl.pk;
     tl.esc += s.status == RASCAS_PK_ESCAPED_;
     tl.abs += s.status == RASCAS_PK_ABSORBED_;
@@ -716,13 +717,14 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// Bounded device work: true (for the whole warp) once this thread has run
-// max_iter loop iterations, the launch has run time_limit_ns, or another warp
-// has raised the abort flag; the first warp to stop raises it.  `iters` is
-// the same in every lane of the warp (the loops are warp-synchronous).
-__device__ __forceinline__ bool out_of_bounds(const Params& P, uint32_t& iters, unsigned long long t0) {
+// Bounded device work: true (for the whole warp) once a lane has done max_iter
+// walk steps (`done`) and asks for more, the launch has run time_limit_ns, or
+// another warp has raised the abort flag; the first warp to stop raises it.
+// `iters` counts the loop's iterations, the same in every lane of the warp (the
+// loops are warp-synchronous).
+__device__ __forceinline__ bool out_of_bounds(const Params& P, uint32_t& iters, uint32_t done, unsigned long long t0) {
     ++iters;
-    bool stop = P.max_iter != 0u && iters > P.max_iter;
+    bool stop = P.max_iter != 0u && done >= P.max_iter;
     if ((iters & 255u) == 0u) {
         if (*(volatile unsigned int*)P.abort_flag != 0u) stop = true;
         if (P.time_limit_ns != 0ull && global_ns() - t0 > P.time_limit_ns) stop = true;
@@ -780,10 +782,13 @@ k_propagate(const __grid_constant__ Params P, PacketsIn in, PacketsOut out, Trac
         s.cc.u0mask = 0u;
         s.halt = false;
         P.save_flag[gt] = 0;
+        tl.spent = 0u - (uint32_t)s.nsteps;   // its steps of earlier rounds do not count in this one
         have = true;
     }
     for (;;) {
-        if (P.limits && out_of_bounds(P, iters, t0)) {
+        // steps, not iterations: a lane that waits for company (served) spends
+        // nothing, and one that has no more work is not asked
+        if (P.limits && out_of_bounds(P, iters, !have && drained ? 0u : tl.spent + (have ? (uint32_t)s.nsteps : 0u), t0)) {
             // a limit was reached: the packet in flight stays unfinished
             if (have && s.status != RASCAS_PK_ACTIVE_)
                 finish_packet<NL>(P, BATCH ? P.models[s.mi] : P.g, s, out, tl);
@@ -1192,7 +1197,7 @@ __global__ void __launch_bounds__(128, ADJ ? 3 : 5) k_peel(const Params* __restr
     uint32_t iters = 0;
     const unsigned long long t0 = P.limits ? global_ns() : 0ull;
     for (;;) {
-        if (P.limits && out_of_bounds(P, iters, t0)) break;
+        if (P.limits && out_of_bounds(P, iters, iters, t0)) break;
         const bool want = !active && !drained;
         const unsigned m = __ballot_sync(kFull, want);
         if (m) {
