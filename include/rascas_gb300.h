@@ -214,7 +214,8 @@ int rascas_set_stream(rascas_ctx *ctx, void *stream);
  *      lines, domain, sources, peeling directions) -----------------------
  * Set-up calls copy their arguments into the context (the caller keeps its
  * structs) and return RASCAS_E_ARG for out-of-range values without changing
- * the context.  They may be called in any order before the first run and
+ * the context; one that runs out of device memory (RASCAS_E_OOM) leaves it
+ * without what the call was to replace.  They may be called in any order before the first run and
  * again between runs; rascas_propagate and the calls after it need the
  * octree, domain, lines and physics (RASCAS_E_STATE otherwise). */
 

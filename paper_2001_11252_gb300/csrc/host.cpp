@@ -378,6 +378,9 @@ int rascas_load_octree(rascas_ctx* ctx, const rascas_octree* t, int mem) {
     if (ce != cudaSuccess) return cuda_fail(ctx, ce, "load_octree");
     if (err) return fail(ctx, RASCAS_E_ARG, err);
     mesh_flags(M, ctx->has_domain ? &ctx->dom : nullptr);
+    // the buffers of the old tree go first: a call that fails from here on
+    // leaves the context without one
+    ctx->has_mesh = false;
     CK(ctx->d_rec.ensure(M.rec.size() * 4));
     CK(ctx->d_son.ensure(M.son.size() * 4));
     CK(ctx->d_nbr.ensure(M.nbr.size() * 4));
@@ -550,7 +553,15 @@ int rascas_set_detector(rascas_ctx* ctx, const rascas_detector* d) {
     if (d->nbin < 1 || !(d->nu_hi > d->nu_lo) || d->ndir < 0 || d->ndir > RASCAS_MAX_DIRS || d->npix < 0 ||
         (d->npix > 0 && !(d->fov > 0)))
         return fail(ctx, RASCAS_E_ARG, "detector: bad values");
+    auto norm2 = [&](int i) {
+        return d->dirs[i][0] * d->dirs[i][0] + d->dirs[i][1] * d->dirs[i][1] + d->dirs[i][2] * d->dirs[i][2];
+    };
+    for (int i = 0; i < d->ndir; ++i)
+        if (!(norm2(i) > 0)) return fail(ctx, RASCAS_E_ARG, "detector: zero direction");
     CK(cudaSetDevice(ctx->device));
+    // the old tallies' buffers and shapes go first: a call that fails from here
+    // on leaves the context without a detector
+    ctx->has_det = false;
     ctx->det = *d;
     Params& P = ctx->P;
     P.g.nu_lo = d->nu_lo;
@@ -562,9 +573,7 @@ int rascas_set_detector(rascas_ctx* ctx, const rascas_detector* d) {
     P.fov = d->npix > 0 ? d->fov : 1.0;
     for (int ax = 0; ax < 3; ++ax) P.img_c[ax] = d->centre[ax];
     for (int i = 0; i < d->ndir; ++i) {
-        double n2 = d->dirs[i][0] * d->dirs[i][0] + d->dirs[i][1] * d->dirs[i][1] + d->dirs[i][2] * d->dirs[i][2];
-        if (!(n2 > 0)) return fail(ctx, RASCAS_E_ARG, "detector: zero direction");
-        double nn = std::sqrt(n2);
+        double nn = std::sqrt(norm2(i));
         double n[3] = {d->dirs[i][0] / nn, d->dirs[i][1] / nn, d->dirs[i][2] / nn};
         for (int ax = 0; ax < 3; ++ax) {
             P.dirs[i][ax] = n[ax];
@@ -1114,6 +1123,7 @@ int rascas_load_batch(rascas_ctx* ctx, const rascas_model* models, int32_t nmode
         }
         cost[m] = t * md.domain.size * M.box_cm;
     }
+    B.nmodels = 0;   // the old batch's buffers go first: none is loaded if the call fails from here on
     B.order.resize(nmodels);
     for (int m = 0; m < nmodels; ++m) B.order[m] = m;
     std::stable_sort(B.order.begin(), B.order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
