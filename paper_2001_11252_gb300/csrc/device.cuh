@@ -62,7 +62,7 @@ static __device__ __noinline__ uint4 philox_block(uint32_t blk, uint32_t id0, ui
 // the lanes of a warp always hit distinct banks).  top_up(), called where the
 // warp is converged, computes the next blocks of every lane together (three
 // blocks interleaved for instruction-level parallelism) and leaves at least
-// the 11 words that a step draws when its first rejection trial succeeds, so
+// the kStepWords that a step draws when its first rejection trial succeeds, so
 // word() reads without asking; need() is called where a draw may go beyond
 // (a second trial, a packet's first draw).  A check and a call to philox_block
 // behind each word kept the compiler from moving loads and functions across
@@ -71,9 +71,21 @@ static __device__ __noinline__ uint4 philox_block(uint32_t blk, uint32_t id0, ui
 // 150000 packets, 118 -> 97 ms; slab, 2000 packets, 212 -> 172 ms.
 // Rows are kCols words apart whatever the block size, so that the address of
 // a row is a constant offset.  Dynamic shared memory of a kernel using Rng
-// starts with kRing rows for the rings.
+// starts with kRing rows for the rings.  A batch launched in blocks of 32
+// threads takes the rows of 128 all the same: 11 and 9 blocks per SM with three
+// and four lines where 16 would fit (200 000 packets, four lines: 9.6 ms, 8.7 in
+// blocks of 64 or more).  Rings and coefficients packed by warp make that 8.7 too,
+// but every block size 1.5-2.5 % slower with three and four lines.
 constexpr uint32_t kRing = 16;
 constexpr uint32_t kCols = 128;   // threads per block, at most
+// Words that a walk step may draw without asking: which absorber 1, decay
+// channel 1, one trial of u_par 3, u_perp 2, phase function 2, next tau 2.  A draw
+// added to a step belongs here too: word() reads whatever the ring holds.
+constexpr uint32_t kTrialWords = 3;
+constexpr uint32_t kAfterTrialWords = 2 + 2 + 2;
+constexpr uint32_t kStepWords = 1 + 1 + kTrialWords + kAfterTrialWords;
+static_assert(kStepWords <= kRing - 4u, "top_up leaves at least kRing - 4 words");
+static_assert(kTrialWords + kAfterTrialWords <= kRing - 3u, "need() reaches kRing - 3 words at most");
 
 struct Rng {
     uint32_t k0, k1, id0, id1;
@@ -313,7 +325,7 @@ __device__ __forceinline__ float sample_upar(Rng& rng, float x, float a, const U
         float u = b1 ? xa - q : xa + q;
         float lim = b1 ? 0.0f : u0sq;
         if (r3 <= expf(__fmaf_rn(-u, u, lim))) return sg * u;
-        rng.need(9);   // another trial and the six draws after it
+        rng.need(kTrialWords + kAfterTrialWords);
     }
     err = true;
     return 0.0f;
