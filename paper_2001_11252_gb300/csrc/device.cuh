@@ -542,7 +542,8 @@ __device__ __forceinline__ bool next_leaf(const Geo& G, const double p[3], const
 // of it, or a link that does not fit, is looked up from the top grid.
 // Against next_leaf: peeling 2^16 packets through the galaxy (2e6 leaves)
 // 55.6 -> 52.4 ms; 2^20 rays the same until the FP64 work went down too.
-// son_loads and nbor_loads count what next_leaf would have read.
+// son_loads and nbor_loads count the reads of next_leaf, whatever is read here:
+// a run's statistics stay those of the neighbour search of Sect. 4.3.
 __device__ __forceinline__ bool linked_leaf(const Geo& G, const double p[3], const double k[3], int axis, Where& w,
                                             int lk, uint32_t& son_loads, uint32_t& nbor_loads) {
     const int L = G.max_level, l = w.level, sh = L - l;
@@ -559,12 +560,28 @@ __device__ __forceinline__ bool linked_leaf(const Geo& G, const double p[3], con
     const int from = axis == 0 ? w.i : (axis == 1 ? w.j : w.k);
     const bool father = ((from & 1) != 0) != up && l >= 1;   // the cell across the face has the same father
     const bool holds = (t[0] >> sh) == c0 && (t[1] >> sh) == c1 && (t[2] >> sh) == c2;
-    if (!father && l >= 2) ++nbor_loads;
     if (!holds || lk == kLinkNone) {
+        const Where from_leaf = w;
         uint32_t loads = 0;
-        ++son_loads;
-        return locate(G, t[0], t[1], t[2], w, loads);
+        locate(G, t[0], t[1], t[2], w, loads);
+        // next_leaf looks in the father, then in the father's neighbour across
+        // the face (or the leaf that covers it), then from the top grid
+        int m = l;
+        bool in = (t[0] >> (sh + 1)) == from_leaf.i >> 1 && (t[1] >> (sh + 1)) == from_leaf.j >> 1 &&
+                  (t[2] >> (sh + 1)) == from_leaf.k >> 1;
+        if (!in && l >= 2) {
+            ++nbor_loads;
+            m = min(w.level, l - 1);
+            const int up_to = L - m, d = l - 1 - m, mask = (1 << (l - 1)) - 1;
+            const int f0 = axis == 0 ? ((from_leaf.i >> 1) + step) & mask : from_leaf.i >> 1;
+            const int f1 = axis == 1 ? ((from_leaf.j >> 1) + step) & mask : from_leaf.j >> 1;
+            const int f2 = axis == 2 ? ((from_leaf.k >> 1) + step) & mask : from_leaf.k >> 1;
+            in = (t[0] >> up_to) == f0 >> d && (t[1] >> up_to) == f1 >> d && (t[2] >> up_to) == f2 >> d;
+        }
+        son_loads += in ? 1u + (uint32_t)(w.level - m) : loads;
+        return true;
     }
+    if (!father && l >= 2) ++nbor_loads;
     if (lk >= 0) {
         const int coarser = lk & 1;
         const int s = sh + coarser;
