@@ -53,6 +53,9 @@ struct HostMesh {
     std::vector<int> son, nbr, top;   // 8 per oct, 8 per oct, 4 per top-grid region
     std::vector<float> rec;           // 8 per leaf
     std::vector<int> leaf_level, leaf_ijk;
+    // of the fields as loaded, for the launch shape: largest n^2 / T of H I and of
+    // the metal, highest T, widest range of a velocity component (cm/s)
+    double n2_over_T[2] = {0.0, 0.0}, T_max = 0.0, v_span = 0.0;
 };
 
 }  // namespace
@@ -288,6 +291,16 @@ const char* build_mesh(const rascas_octree* t, int mem, HostMesh& M, cudaError_t
     for (int i = 0; i < nleaf; ++i) {
         float* r = &M.rec[8 * (size_t)i];
         for (int j = 0; j < 7; ++j) r[j] = f[j][i];
+    }
+    for (int i = 0; i < nleaf; ++i) {
+        const double T = std::fmax((double)f[4][i], 1e-30);
+        M.n2_over_T[0] = std::fmax(M.n2_over_T[0], (double)f[0][i] * f[0][i] / T);
+        M.n2_over_T[1] = std::fmax(M.n2_over_T[1], (double)f[6][i] * f[6][i] / T);
+        M.T_max = std::fmax(M.T_max, T);
+    }
+    for (int j = 1; j <= 3; ++j) {
+        const auto lim = std::minmax_element(f[j].begin(), f[j].end());
+        M.v_span = std::fmax(M.v_span, (double)*lim.second - (double)*lim.first);
     }
     M.noct = noct;
     M.nleaf = nleaf;
@@ -657,6 +670,36 @@ int persistent_grid(rascas_ctx* ctx, bool peel) {
     return ctx->sms * per_sm;
 }
 
+// Warps that few packets are spread over, one lane each, then two, and so on.  A
+// warp issues every branch that any of its lanes takes, so a packet with fewer
+// neighbours runs faster, and a launch is as long as its longest packet; but
+// every warp puts its FP64 instructions through the SM's one FP64 pipe, whether
+// for one lane or 32.  So long histories want many warps, short ones few:
+//                                            full warps  1/SM   3/SM   8/SM  16/SM
+//   slab, tau0 = 2000, 2000 packets (ms)            236   204    180    179    173
+//   slab, tau0 = 1000, 10000 packets (ms)           183   177    176    153    158
+//   peeled galaxy, 3 lines, 5000 packets (ms)      4.25  4.27   3.40   2.94   2.67
+//   deuterium sphere, 10000 packets (ms)           25.5  25.7   25.1   26.0   24.6
+//   outflow, tau0 = 200, 5000 packets (us)          168   176    189    199    199
+//   Mg II wind, tau0 = 100, 10000 packets (us)      332   337    346    406    397
+//   Fe II wind, tau0 = 100, 3000 packets (us)       259   258    304    308    313
+// Histories are short where the gas moves by many thermal widths and has less
+// than two optical depths at line centre per thermal width of that range (the
+// last three; 2.3 such depths already want 8), unless each event is peeled.
+// Eight warps per SM otherwise, three with several lines, which cost more FP64
+// per step, and no peeling (Fe II, tau0 = 1e4, 6000 packets: 387 us, 404 with 8).
+int spread_warps(const rascas_ctx* ctx, const Params& P, const HostMesh* M) {
+    if (M && P.ndir == 0) {
+        double tau = 0.0;   // at most, from the domain's centre to its border
+        for (int i = 0; i < P.nline; ++i)
+            tau = std::fmax(tau, std::sqrt(M->n2_over_T[P.line[i].dens == 1]) * P.line[i].abund * P.line[i].sig_pref);
+        tau *= ctx->dom.size * M->box_cm;
+        const double widths = M->v_span / (P.line[0].vth_pref * std::sqrt(M->T_max));
+        if (widths >= 32.0 && tau < 2.0 * widths) return ctx->sms;
+    }
+    return ctx->sms * (P.nline == 1 || P.ndir > 0 ? 8 : 3);
+}
+
 int run_propagate(rascas_ctx* ctx, const rascas_packets_in* in, int64_t n, const rascas_packets_out* out,
                   int mem, rascas_run_stats* stats, rascas_event* events, int32_t* nevents, int32_t max_events,
                   bool tallies, const Params* adj = nullptr) {
@@ -675,6 +718,7 @@ int run_propagate(rascas_ctx* ctx, const rascas_packets_in* in, int64_t n, const
             P.g.nu_range = 1.0;
         }
     }
+    P.spread = spread_warps(ctx, P, &ctx->mesh);
     rg::PacketsIn din{in->pos, in->dir, in->nu, in->id, (long long)n, 0};
     rg::PacketsOut dout{};
     if (out) dout = rg::PacketsOut{out->status, out->nscatt, out->nu, out->pos, out->dir, out->path};
@@ -1037,6 +1081,7 @@ int rascas_propagate_noalloc(rascas_ctx* ctx, const rascas_packets_in* in, int64
     Params P = ctx->P;
     P.g.spec = nullptr;   // per-packet outputs only: no tallies, no peeling
     P.ndir = 0;
+    P.spread = spread_warps(ctx, P, &ctx->mesh);
     P.counters = cnt_d;
     P.head = cnt_d + rg::CNT_N;
     P.abort_flag = (unsigned int*)(cnt_d + rg::CNT_N + 1);
@@ -1236,6 +1281,7 @@ int run_batch(rascas_ctx* ctx, int32_t mode, const rg::PacketsOut& out, rascas_r
     P.model_first = (const long long*)B.d_first.p;
     P.nmodels = B.nmodels;
     P.refill = B.refill;
+    P.spread = spread_warps(ctx, P, nullptr);
     rg::PacketsIn in{(const double*)B.d_pos.p, (const double*)B.d_dir.p, (const double*)B.d_nu.p,
                      (const uint64_t*)B.d_id.p, B.npackets, 0};
     rg::TraceOut tr{nullptr, nullptr, 0};

@@ -168,7 +168,9 @@ struct Params {
     unsigned int* abort_flag;
     // batch queue: consecutive packets a lane reserves per queue grab
     int refill;
-    // lanes of each warp that take packets (lanes_per_warp)
+    // few packets are spread over this many warps (spread_warps, host side) by
+    // letting only some lanes of each warp take packets (lanes_per_warp)
+    int spread;
     int lanes;
     unsigned wait;   // iterations that a lane may wait for company before a long piece of the loop
     // run scratch

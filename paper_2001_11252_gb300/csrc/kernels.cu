@@ -1483,18 +1483,8 @@ static cudaError_t launch_nl(const Params& P_, const PacketsIn& in, const Packet
                              int grid, int block, cudaStream_t st) {
     size_t smem = smem_bytes(NL, block);
     Params P = P_;
-    // Few packets: a lane each in some of the resident warps, then two lanes
-    // each, and so on.  A warp issues every branch that any of its lanes takes,
-    // so a packet with fewer neighbours runs faster, and its launch is as long as
-    // its longest packet; but every warp puts its FP64 instructions through the
-    // SM's one FP64 pipe, whether for one lane or 32.  With one line eight warps
-    // per SM: 2000 packets in a slab (longest: 86 409 scatterings) 269 ms in full
-    // warps, 226 with 8 lanes, 212 with 4, 204 with 2, 205 with 1.  With several
-    // lines, which cost more FP64 per step and have short histories where they
-    // fluoresce, three: 10000 packets, Mg II wind, 351 us, 409 with eight warps
-    // per SM (352 in full warps); 5000 packets peeled through the galaxy 3.4 ms,
-    // 3.0 with eight (4.2 in full warps).
-    P.lanes = lanes_per_warp(in.n - in.first, (long long)grid * block / 32 * (NL == 1 ? 8 : 3) / 16);
+    // few packets: a lane each in some of the warps, then two lanes each, and so on
+    P.lanes = lanes_per_warp(in.n - in.first, std::min((long long)grid * block / 32, (long long)P.spread));
     P.wait = in.n - in.first < (long long)grid * block ? 1u : 4u;
     // per-event traces are recorded by single-model runs without peeling only
     if (tr.nev && (P.nmodels > 0 || P.ndir > 0)) return cudaErrorInvalidValue;
