@@ -53,7 +53,7 @@ struct HostMesh {
     std::vector<int> son, nbr, top;   // 8 per oct, 8 per oct, 4 per top-grid region
     std::vector<float> rec;           // 8 per leaf
     std::vector<int> leaf_level, leaf_ijk;
-    // of the fields as loaded, for the launch shape: largest n^2 / T of H I and of
+    // of the fields as loaded (a sample of the leaves), for the launch shape: largest n^2 / T of H I and of
     // the metal, highest T, widest range of a velocity component (cm/s)
     double n2_over_T[2] = {0.0, 0.0}, T_max = 0.0, v_span = 0.0;
 };
@@ -292,16 +292,21 @@ const char* build_mesh(const rascas_octree* t, int mem, HostMesh& M, cudaError_t
         float* r = &M.rec[8 * (size_t)i];
         for (int j = 0; j < 7; ++j) r[j] = f[j][i];
     }
-    for (int i = 0; i < nleaf; ++i) {
+    // some 2^14 leaves tell enough (all of 1e6 would make the load 13 % longer)
+    const int step = std::max(1, nleaf >> 14);
+    double lo[3], hi[3];
+    for (int j = 0; j < 3; ++j) lo[j] = hi[j] = f[1 + j][0];
+    for (int i = 0; i < nleaf; i += step) {
         const double T = std::fmax((double)f[4][i], 1e-30);
         M.n2_over_T[0] = std::fmax(M.n2_over_T[0], (double)f[0][i] * f[0][i] / T);
         M.n2_over_T[1] = std::fmax(M.n2_over_T[1], (double)f[6][i] * f[6][i] / T);
         M.T_max = std::fmax(M.T_max, T);
+        for (int j = 0; j < 3; ++j) {
+            lo[j] = std::fmin(lo[j], (double)f[1 + j][i]);
+            hi[j] = std::fmax(hi[j], (double)f[1 + j][i]);
+        }
     }
-    for (int j = 1; j <= 3; ++j) {
-        const auto lim = std::minmax_element(f[j].begin(), f[j].end());
-        M.v_span = std::fmax(M.v_span, (double)*lim.second - (double)*lim.first);
-    }
+    for (int j = 0; j < 3; ++j) M.v_span = std::fmax(M.v_span, hi[j] - lo[j]);
     M.noct = noct;
     M.nleaf = nleaf;
     M.max_level = max_level;
@@ -675,17 +680,19 @@ int persistent_grid(rascas_ctx* ctx, bool peel) {
 // neighbours runs faster, and a launch is as long as its longest packet; but
 // every warp puts its FP64 instructions through the SM's one FP64 pipe, whether
 // for one lane or 32.  So long histories want many warps, short ones few:
-//                                            full warps  1/SM   3/SM   8/SM  16/SM
-//   slab, tau0 = 2000, 2000 packets (ms)            236   204    180    179    173
-//   slab, tau0 = 1000, 10000 packets (ms)           183   177    176    153    158
-//   peeled galaxy, 3 lines, 5000 packets (ms)      4.25  4.27   3.40   2.94   2.67
-//   deuterium sphere, 10000 packets (ms)           25.5  25.7   25.1   26.0   24.6
-//   outflow, tau0 = 200, 5000 packets (us)          168   176    189    199    199
-//   Mg II wind, tau0 = 100, 10000 packets (us)      332   337    346    406    397
-//   Fe II wind, tau0 = 100, 3000 packets (us)       259   258    304    308    313
+//                                            full warps  1/SM   2/SM   3/SM   8/SM  16/SM
+//   slab, tau0 = 2000, 2000 packets (ms)            236   204    182    180    179    173
+//   slab, tau0 = 1000, 10000 packets (ms)           183   177    181    176    153    158
+//   peeled galaxy, 3 lines, 5000 packets (ms)      4.25  4.27   3.70   3.40   2.94   2.67
+//   deuterium sphere, 10000 packets (ms)           25.5  25.7   24.3   25.1   26.0   24.6
+//   outflow, tau0 = 200, 5000 packets (us)          168   176    179    189    199    199
+//   Mg II wind, tau0 = 100, 10000 packets (us)      332   337    333    346    406    397
+//   the same, 1000 packets (us)                     266   265    249    248    262    261
+//   Fe II wind, tau0 = 100, 3000 packets (us)       259   258    276    304    308    313
 // Histories are short where the gas moves by many thermal widths and has less
 // than two optical depths at line centre per thermal width of that range (the
-// last three; 2.3 such depths already want 8), unless each event is peeled.
+// last four: two warps per SM; 2.3 such depths already want 8), unless each event
+// is peeled.
 // Eight warps per SM otherwise, three with several lines, which cost more FP64
 // per step, and no peeling (Fe II, tau0 = 1e4, 6000 packets: 387 us, 404 with 8).
 int spread_warps(const rascas_ctx* ctx, const Params& P, const HostMesh* M) {
@@ -695,7 +702,7 @@ int spread_warps(const rascas_ctx* ctx, const Params& P, const HostMesh* M) {
             tau = std::fmax(tau, std::sqrt(M->n2_over_T[P.line[i].dens == 1]) * P.line[i].abund * P.line[i].sig_pref);
         tau *= ctx->dom.size * M->box_cm;
         const double widths = M->v_span / (P.line[0].vth_pref * std::sqrt(M->T_max));
-        if (widths >= 32.0 && tau < 2.0 * widths) return ctx->sms;
+        if (widths >= 32.0 && tau < 2.0 * widths) return 2 * ctx->sms;
     }
     return ctx->sms * (P.nline == 1 || P.ndir > 0 ? 8 : 3);
 }
