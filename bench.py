@@ -48,10 +48,10 @@ PIPE_PER_SCATT = {"fma": 2821713684031 / 111923728554, "fp64": 59794947584 / 111
                   "xu": 169162376323 / 111923728554}
 # DRAM bytes per leaf visit of k_ray_tau on the synthetic galaxy
 # (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of 2^18
-# rays from emitting leaves, 59 732 805 leaf visits, with the neighbour search
-# by records; the walk by face links moved 46.6 bytes per visit through a
-# galaxy of 3.2e6 leaves)
-RAY_DRAM_BYTES_PER_VISIT = (4.107982e9 + 49.11232e6) / 59732805
+# rays from emitting leaves, 59 732 805 leaf visits: a leaf's record and its
+# face links, 64 bytes, and what the sectors of the top grid and of refined
+# neighbours add; a smaller galaxy of 3.2e6 leaves moves 46.6 per visit)
+RAY_DRAM_BYTES_PER_VISIT = (5.965077504e9 + 21.89824e6) / 59732805
 
 
 def parse():

@@ -184,6 +184,11 @@ typedef struct {
     double *nu, *pos, *dir, *path;
 } rascas_packets_out;
 
+/* Counts of a run.  upar_trials: rejection trials of u_par.  leaf_loads: leaf
+ * records taken up, by packets and peeling rays.  son_loads, nbor_loads: reads of
+ * the son array (and of the top grid) and of neighbour records that the search of
+ * Sect. 4.3 makes for the leaves crossed; peeling rays count them as packets do,
+ * though they follow face links and read fewer. */
 typedef struct {
     int64_t packets, escaped, absorbed, capped, errors;
     int64_t nscatt_line, nscatt_dust, ncross, npeel_rays, npeel_cells;

@@ -945,10 +945,10 @@ __device__ __forceinline__ void ray_load(const RayInit* __restrict__ in, long lo
 
 // Persistent walk: each lane walks one ray leaf by leaf and takes the next ray
 // from the queue head as soon as its ray is done, so the lanes of a warp stay
-// busy whatever the spread of ray lengths.  Six blocks per SM (80 registers, no
-// spills): 2^20 rays of 153 leaves through the galaxy in 7.6 ms, 7.8 with eight
-// blocks (64 registers); 9.5 ms with next_leaf and face_distance (the walk of
-// the scattering kernel), eight blocks.
+// busy whatever the spread of ray lengths.  Six blocks per SM (80 registers; three
+// lines spill 4 bytes, four 10): 2^20 rays of 153 leaves through the galaxy, three
+// lines, in 7.5 ms, 7.8 with eight blocks (64 registers); 9.5 ms with next_leaf
+// and face_distance (the walk of the scattering kernel), eight blocks.
 template <int NL>
 __global__ void __launch_bounds__(128, 6) k_ray_tau(const Params* __restrict__ G, long long n,
                                                  const RayInit* __restrict__ init, double* tau, int32_t* cells,
@@ -1041,8 +1041,10 @@ __device__ __forceinline__ bool floor_certain(float t, float err, float& fl) {
 // spectrum channel (or -1) and image pixel (or -1) of a peeled contribution:
 // the plain definitions' operations in FP64, unfused (exact ties bin as in the
 // oracle), where FP32 does not already decide the bin.  The plain form of a
-// record takes some 70 FP64 instructions, three divisions among them; all but
-// about one record in a thousand end with four subtractions.  With the merged
+// record takes some 70 FP64 instructions, three divisions among them; most end
+// with four subtractions.  The share that does not grows with the pixels along a
+// side, by about 1.5e-5 for each: two records in a thousand at 100 x 100 pixels,
+// 6 % at 4096 x 4096, where most warps hold one.  With the merged
 // reservation, outflow of 30000 packets (1.6e8 rays): 204 -> 176 ms, the prep
 // pass 25.9 -> 11.5 ms of it.
 __device__ __forceinline__ void peel_bins(const Params& P, const PeelRec& q, int& ch, long long& px) {
@@ -1414,8 +1416,6 @@ __global__ void k_leaf_links(Geo g, int* __restrict__ link) {
             }
             out[face] = lk;
         }
-        out[6] = level;
-        out[7] = 0;
     }
 }
 
